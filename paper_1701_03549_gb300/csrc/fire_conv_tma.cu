@@ -1,27 +1,16 @@
-// TMA-fed implicit-GEMM convolution for the surrogate's 128 -> 128 layers
-// (forward and input gradient), on tcgen05 tensor cores.
+// TMA-fed implicit-GEMM convolutions of the surrogate network on tcgen05
+// tensor cores: the 128 -> 128 layers forward and input gradient
+// (k_conv_pair), their weight gradient (k_wgrad_tma) and the first layer
+// forward (k_conv1_tma).
 //
-// A CTA computes a 128-pixel x 128-channel tile.  The K loop runs over the
-// 9 taps x 2 halves of 64 input channels; for each 64-wide slab
-//   * one thread issues two TMA loads: the activation tile, shifted by the
-//     tap's offset, through a 4-D tensor map over the NHWC buffer (channels,
-//     x, y, sample) whose out-of-range elements read as zero (the zero
-//     padding of the convolution), and the 128 x 64 weight slab through a 2-D
-//     map; both land 128-byte swizzled, which is the canonical K-major
-//     SWIZZLE_128B operand layout of the tensor core;
-//   * another thread waits for the slab, issues four 128 x 128 x 16 MMAs into
-//     the tensor-memory accumulator and commits them to the slab's "empty"
-//     barrier, which hands the stage back to the loader.
-// k_conv_tma runs one tile per CTA: two stages (64 KB) let three CTAs share
-// an SM, so the epilogues of some (tensor memory -> registers -> bias/ReLU or
-// ReLU mask -> BF16 stores) overlap the main loops of the others.
-// k_conv_tma_p, the default, is persistent: two CTAs per SM loop over tiles
-// with three stages and two tensor-memory accumulators, the loads and MMAs
-// of the next tile overlapping the epilogue of the previous one within the
-// CTA (on a GB300, 9 % more training throughput than k_conv_tma; a single
-// persistent CTA per SM was slower than either).  Every wait is bounded; on a
-// timeout the CTA records an error, waits (bounded) for its own copies and
-// MMAs in flight, frees its tensor memory and returns.
+// In each, one thread issues tensor-map copies of shifted NHWC activation
+// boxes (channels, x, y, sample; out-of-range elements read as zero, which is
+// the convolution's zero padding) that land swizzled, in the tensor core's
+// canonical layouts; one issues MMAs into a tensor-memory accumulator and
+// commits them to the barriers that hand the stages back; warps drain the
+// accumulator (tensor memory -> registers -> stores).  Every wait is bounded;
+// on a timeout the CTA records an error, waits (bounded) for its own copies
+// and MMAs in flight, frees its tensor memory and returns.
 #include "fire_internal.h"
 #include "fire_tc.cuh"
 
@@ -35,21 +24,9 @@
 namespace fire {
 namespace convtma {
 
-#ifndef FIRE_CONV_STAGES
-#define FIRE_CONV_STAGES 2
-#endif
-#ifndef FIRE_CONV_PERSISTENT
-#define FIRE_CONV_PERSISTENT 1   // 0: one tile per CTA (k_conv_tma)
-#endif
-constexpr int kStages = FIRE_CONV_STAGES;       // shared-memory stages per CTA
 constexpr int kTileBytes = 128 * 128;           // 128 rows x 64 BF16
 constexpr int kStageBytes = 2 * kTileBytes;     // A + B
-constexpr int kSmem = kStages * kStageBytes + 1024;
 constexpr int kSlabs = 18;                      // 9 taps x 2 channel halves
-// CTAs that fit on one SM (227 KB of shared memory; 128 tensor-memory
-// columns each, so at most four).
-constexpr int kCtasPerSm =
-    (227 * 1024) / (kSmem + 2048) > 4 ? 4 : (227 * 1024) / (kSmem + 2048);
 // The weight-gradient kernel's own stage count and residency.
 #ifndef FIRE_WGRAD_STAGES
 #define FIRE_WGRAD_STAGES 2
@@ -117,14 +94,170 @@ __device__ __forceinline__ bool pos16(uint32_t u)
     return !(u & 0x8000u) && (u & 0x7fffu);
 }
 
+// 32 bytes of one row per thread: whole sectors, where 16-byte accesses of
+// rows 256 bytes apart touch every sector twice.
+__device__ __forceinline__ void st_global32(void *p, const uint32_t v[8])
+{
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p),
+                 "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]),
+                 "r"(v[6]), "r"(v[7])
+                 : "memory");
+}
+
+__device__ __forceinline__ void ld_global32(const void *p, uint32_t v[8])
+{
+    asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]),
+                   "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+                 : "l"(p));
+}
+
+// One lane of a converged warp.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(p));
+    return p != 0;
+}
+
+__device__ __forceinline__ bool all_ok(bool ok)
+{
+    return __all_sync(0xffffffffu, ok);
+}
+
+// --- CTA-pair primitives (cta_group::2) -------------------------------------
+
+__device__ __forceinline__ uint32_t cluster_rank()
+{
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\t"
+                 "barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// Address in the shared window of CTA 0 of the pair of a local address.
+__device__ __forceinline__ uint32_t leader_addr(const void *p)
+{
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"(tc::smem_addr(p)));
+    return r;
+}
+
+__device__ __forceinline__ void arrive_cluster(uint32_t cluster_addr)
+{
+    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(
+                     cluster_addr)
+                 : "memory");
+}
+
+// Tensor-map copies into this CTA's shared memory whose bytes count on a
+// barrier of either CTA of the pair.
+__device__ __forceinline__ void tma_4d_pair(uint32_t dst, const CUtensorMap *map,
+                                            int c0, int c1, int c2, int c3,
+                                            uint32_t bar)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.tile."
+        "mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3),
+        "r"(bar)
+        : "memory");
+}
+
+__device__ __forceinline__ void tma_2d_pair(uint32_t dst, const CUtensorMap *map,
+                                            int c0, int c1, uint32_t bar)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile."
+        "mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(bar)
+        : "memory");
+}
+
+__device__ __forceinline__ void mma_bf16_pair(uint32_t d_tmem, uint64_t adesc,
+                                              uint64_t bdesc, uint32_t idesc,
+                                              bool accumulate)
+{
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.u32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(
+            d_tmem),
+        "l"(adesc), "l"(bdesc), "r"(idesc), "r"((uint32_t)accumulate)
+        : "memory");
+}
+
+// Arrives on the barrier at this offset in both CTAs once the MMAs issued so
+// far are done.
+__device__ __forceinline__ void commit_pair(void *bar)
+{
+    asm volatile(
+        "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster."
+        "multicast::cluster.b64 [%0], %1;" ::"r"(tc::smem_addr(bar)),
+        "h"((uint16_t)3)
+        : "memory");
+}
+
+__device__ __forceinline__ void tmem_alloc_pair(uint32_t *dst_smem, uint32_t ncols)
+{
+    asm volatile(
+        "tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+            tc::smem_addr(dst_smem)),
+        "r"(ncols)
+        : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" :::
+                     "memory");
+}
+
+__device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols)
+{
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr),
+                 "r"(ncols)
+                 : "memory");
+}
+
+// How the pair convolution streams a layer's activations (conv_shape): strips
+// of `px` pixels x 64 channels, each serving `taps` taps (the three of a row,
+// or one), in `na` shared-memory stages.
+struct StripShape {
+    int taps, px, na;
+};
+
+constexpr int kWHalf = 64 * 128;                // 64 weight rows x 64 BF16
+constexpr int kWBytes = kSlabs * kWHalf;        // one CTA's half of the weights
+constexpr int kStripRoom = 80 * 1024;
+constexpr int kMaxA = 5;
+constexpr int kEpiWarps = 4;
+constexpr int kPairThreads = 32 * (kEpiWarps + 3);
+constexpr int kPairSmem = kWBytes + kStripRoom + 2048;   // + alignment, barriers
+
+struct PairShared {
+    unsigned long long afull[kMaxA], aempty[kMaxA], wfull[kSlabs];
+    unsigned long long tfull[2], tempty[2], done;
+    uint32_t tmem_slot;
+    int fail, issued, used;
+    float bias[128];
+};
+static_assert(sizeof(PairShared) <= 1024, "barrier area");
+
 // Epilogue of one accumulator row (pixel p, 128 channels in tensor memory at
 // taddr): forward, bias and ReLU; input gradient, zero where the layer
-// below's activation is not positive; BF16 stores.
-__device__ __forceinline__ void conv_epilogue(const Epi &epi, const float *s_bias,
-                                              uint32_t taddr, int p)
+// below's activation (mask) is not positive; BF16 stores.
+__device__ __forceinline__ void pair_epilogue(const Epi &epi, const float *s_bias,
+                                              uint32_t taddr, size_t p,
+                                              const uint32_t mask[64])
 {
-    uint16_t *orow = epi.out + (size_t)p * 128;
-#pragma unroll 1
+    uint16_t *orow = epi.out + p * 128;
+#pragma unroll
     for (int c0 = 0; c0 < 128; c0 += 32) {
         float v[32];
         tc::tmem_ld32(taddr + (uint32_t)c0, v);
@@ -135,289 +268,246 @@ __device__ __forceinline__ void conv_epilogue(const Epi &epi, const float *s_bia
                 pk[j] = pack2(fmaxf(v[2 * j] + s_bias[c0 + 2 * j], 0.0f),
                               fmaxf(v[2 * j + 1] + s_bias[c0 + 2 * j + 1], 0.0f));
         } else {
-            const uint4 *hp =
-                reinterpret_cast<const uint4 *>(epi.hprev + (size_t)p * 128 + c0);
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const uint4 h = hp[q];
-                const uint32_t hw[4] = {h.x, h.y, h.z, h.w};
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const int e = 2 * (4 * q + j);
-                    pk[4 * q + j] = pack2(pos16(hw[j] & 0xffffu) ? v[e] : 0.0f,
-                                          pos16(hw[j] >> 16) ? v[e + 1] : 0.0f);
-                }
+            for (int j = 0; j < 16; ++j) {
+                const uint32_t h = mask[c0 / 2 + j];
+                pk[j] = pack2(pos16(h & 0xffffu) ? v[2 * j] : 0.0f,
+                              pos16(h >> 16) ? v[2 * j + 1] : 0.0f);
             }
         }
-        uint4 *o = reinterpret_cast<uint4 *>(orow + c0);
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-            o[q] = make_uint4(pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
+        st_global32(orow + c0, pk);
+        st_global32(orow + c0 + 16, pk + 8);
     }
 }
 
+// Convolution of a 128 -> 128 layer on CTA pairs (cta_group::2).  The pair
+// computes 256 pixels x 128 channels, each CTA its own 128 pixels (rows of A)
+// with 64 rows of the weights (half of B, read by the tensor cores of both
+// SMs).  The K loop runs over the taps and the two 64-channel halves, in this
+// order.
+//
+// What bounds it, and why this shape (8 x 256 x 256, 154.6 GFLOP a layer):
+//  * half the weights are 144 KB, so they are loaded once and stay: only
+//    activations stream.  Distinct data reaches an SM from L2 at no more than
+//    about 30 bytes per clock when all SMs read (9 TB/s), and a 16 KB box per
+//    tap and half needs 64; a strip of 128 + 2 d pixels that serves the three
+//    taps of a row needs 6 to 8 KB per tap and half.  d = 64 has no room for
+//    three strips and streams a box per tap.
+//  * the issuing thread's own instructions: with waits, commits and
+//    descriptor arithmetic per 64-wide slab it took 500 clocks a slab
+//    whatever the MMA count, against 256 for the slab's MMAs.  Waits and
+//    commits per row of taps, unrolled, leave the tensor core the bound.
+// Measured (one layer, 1909 TFLOP/s measured peak): 90 us for d <= 16 (1718
+// TFLOP/s), 126 us for d = 32 (three strips, one in flight), 135 us for
+// d = 64; one 128-pixel tile per CTA with boxes per tap and streamed weights
+// took 136 us for every d.
+//
+// Persistent: one pair per two SMs walks pairs of tiles.  In both CTAs one
+// thread issues the strip copies, whose bytes count on the leader's barrier
+// (CTA 0), one loads the weights, four warps drain the accumulator; a warp of
+// the leader issues the MMAs into one of two 128-column accumulators, so that
+// a tile's epilogue runs under the next tile's MMAs.
+//
 // sign = +1: forward (source pixel p + off(t)); -1: input gradient (p - off(t)).
-__global__ void __launch_bounds__(128, kCtasPerSm)
-    k_conv_tma(const __grid_constant__ CUtensorMap act,
-               const __grid_constant__ CUtensorMap wts, Epi epi, int S, int lgS,
-               int d, int sign, uint32_t *err)
+// A strip of `px` pixels serves kTaps taps (StripShape); `na` strip stages.
+template <int kTaps>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
+    k_conv_pair(const __grid_constant__ CUtensorMap act,
+                const __grid_constant__ CUtensorMap wts, Epi epi, int px, int na, int S,
+                int lgS, int d, int sign, int npairs, uint32_t *err)
 {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
-    __shared__ __align__(8) unsigned long long full[kStages], empty[kStages], done;
-    __shared__ uint32_t tmem_slot;
-    __shared__ int s_fail, s_issued, s_consumed;
-    __shared__ float s_bias[128];
+    const uint32_t raw = tc::smem_addr(smem_raw);
+    const uint32_t wbase = (raw + 1023u) & ~1023u;
+    const uint32_t abase = wbase + kWBytes;
+    PairShared &sh = *reinterpret_cast<PairShared *>(smem_raw + (wbase - raw) + kWBytes +
+                                                     kStripRoom);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const uint32_t base = (tc::smem_addr(smem_raw) + 1023u) & ~1023u;
-    const int m0 = blockIdx.x * 128;
-    if (epi.mode == 0) s_bias[tid] = epi.bias[tid];
-    const int b = m0 >> (2 * lgS);
-    const int y0 = (m0 >> lgS) & (S - 1), x0 = m0 & (S - 1);
-
-    if (warp == 0) {
-        tc::tmem_alloc(&tmem_slot, 128);
-        tc::tmem_relinquish();
-    }
+    const int rank = (int)cluster_rank();
+    const int pair0 = blockIdx.x >> 1, pstep = gridDim.x >> 1;
+    if (epi.mode == 0 && tid < 128) sh.bias[tid] = epi.bias[tid];
+    if (warp == kEpiWarps) tmem_alloc_pair(&sh.tmem_slot, 256);
     if (tid == 0) {
-        for (int i = 0; i < kStages; ++i) {
-            tc::mbar_init(&full[i], 1);
-            tc::mbar_init(&empty[i], 1);
+        for (int i = 0; i < kMaxA; ++i) {
+            tc::mbar_init(&sh.afull[i], 1);
+            tc::mbar_init(&sh.aempty[i], 1);
         }
-        tc::mbar_init(&done, 1);
-        s_fail = 0;
-        s_issued = 0;
-        s_consumed = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    tc::fence_before_sync();
-    __syncthreads();
-    tc::fence_after_sync();
-    const uint32_t tmem = tmem_slot;
-
-    if (warp == 0 && lane == 0) {
-        // loader
-        int s = 0;
-        for (; s < kSlabs; ++s) {
-            const int st = s % kStages;
-            if (s >= kStages &&
-                !tc::mbar_wait_bounded(&empty[st], ((s / kStages) - 1) & 1)) {
-                atomicOr(&s_fail, 1);
-                break;
-            }
-            if (*(volatile int *)&s_fail) break;
-            const int tap = s >> 1, c0 = (s & 1) * 64;
-            const int dy = sign * (tap / 3 - 1) * d, dx = sign * (tap % 3 - 1) * d;
-            const uint32_t sa = base + st * kStageBytes;
-            expect_tx(&full[st], kStageBytes);
-            tma_4d(sa, &act, c0, x0 + dx, y0 + dy, b, &full[st]);
-            tma_2d(sa + kTileBytes, &wts, s * 64, 0, &full[st]);
-        }
-        s_issued = s;
-    } else if (warp == 1 && lane == 0) {
-        // MMA issuer
-        constexpr uint32_t idesc = tc::idesc_bf16(128, 128);
-        int s = 0;
-        for (; s < kSlabs; ++s) {
-            const int st = s % kStages;
-            if (!tc::mbar_wait_bounded(&full[st], (s / kStages) & 1)) {
-                atomicOr(&s_fail, 1);
-                break;
-            }
-            tc::fence_after_sync();
-            const uint32_t sa = base + st * kStageBytes, sb = sa + kTileBytes;
-#pragma unroll
-            for (int kk = 0; kk < 4; ++kk)
-                tc::mma_bf16(tmem, desc_sw128(sa + kk * 32), desc_sw128(sb + kk * 32),
-                             idesc, s > 0 || kk > 0);
-            tc::mma_commit(&empty[st]);
-        }
-        s_consumed = s;
-        if (s == kSlabs) tc::mma_commit(&done);
-    }
-    __syncwarp();
-    if (!tc::mbar_wait_bounded(&done, 0)) atomicOr(&s_fail, 1);
-    __syncthreads();
-    tc::fence_after_sync();
-
-    if (!s_fail) {
-        conv_epilogue(epi, s_bias, tmem + ((uint32_t)(warp * 32) << 16),
-                      m0 + warp * 32 + lane);
-    } else if (tid == 0) {
-        atomicOr(err, 1u);
-        // copies issued but never consumed must land before the CTA leaves
-        for (int s = s_consumed; s < s_issued; ++s)
-            tc::mbar_wait_bounded(&full[s % kStages], (s / kStages) & 1);
-    }
-    tc::fence_before_sync();
-    __syncthreads();
-    if (warp == 0) tc::tmem_dealloc(tmem, 128);
-}
-
-// Persistent variant of k_conv_tma: two CTAs per SM, each looping over tiles
-// (tile = blockIdx.x, blockIdx.x + gridDim.x, ...) with three shared-memory
-// stages and two 128-column tensor-memory accumulators, so that the next
-// tile's loads and MMAs run while the previous tile's epilogue drains its
-// accumulator.  Warp 0 (one thread) issues the TMA loads, warp 1 (one thread)
-// the MMAs, warps 2..5 run the epilogue (warp w reads tensor-memory lanes
-// 32 (w mod 4) .. 32 (w mod 4) + 31, as tcgen05.ld requires).  Every wait is
-// bounded; on a timeout the CTA records an error, lets its copies and MMAs in
-// flight finish (bounded), frees its tensor memory and returns.
-constexpr int kPStages = 3;
-constexpr int kPSmem = kPStages * kStageBytes + 1024;
-constexpr int kPThreads = 192;
-
-__device__ __forceinline__ void mbar_arrive(void *bar)
-{
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(
-                     tc::smem_addr(bar))
-                 : "memory");
-}
-
-__global__ void __launch_bounds__(kPThreads, 2)
-    k_conv_tma_p(const __grid_constant__ CUtensorMap act,
-                 const __grid_constant__ CUtensorMap wts, Epi epi, int S, int lgS,
-                 int d, int sign, int ntiles, uint32_t *err)
-{
-    extern __shared__ __align__(1024) unsigned char smem_raw[];
-    __shared__ __align__(8) unsigned long long full[kPStages], empty[kPStages];
-    __shared__ __align__(8) unsigned long long tfull[2], tempty[2], done;
-    __shared__ uint32_t tmem_slot;
-    __shared__ int s_fail, s_issued, s_consumed;
-    __shared__ float s_bias[128];
-
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const uint32_t base = (tc::smem_addr(smem_raw) + 1023u) & ~1023u;
-    if (epi.mode == 0 && tid < 128) s_bias[tid] = epi.bias[tid];
-    if (warp == 0) {
-        tc::tmem_alloc(&tmem_slot, 256);
-        tc::tmem_relinquish();
-    }
-    if (tid == 0) {
-        for (int i = 0; i < kPStages; ++i) {
-            tc::mbar_init(&full[i], 1);
-            tc::mbar_init(&empty[i], 1);
-        }
+        for (int i = 0; i < kSlabs; ++i) tc::mbar_init(&sh.wfull[i], 1);
         for (int i = 0; i < 2; ++i) {
-            tc::mbar_init(&tfull[i], 1);
-            tc::mbar_init(&tempty[i], 128);   // every epilogue thread arrives
+            tc::mbar_init(&sh.tfull[i], 1);
+            tc::mbar_init(&sh.tempty[i], 2 * kEpiWarps);   // of both CTAs
         }
-        tc::mbar_init(&done, 1);
-        s_fail = 0;
-        s_issued = 0;
-        s_consumed = 0;
+        tc::mbar_init(&sh.done, 1);
+        sh.fail = 0;
+        sh.issued = sh.used = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     tc::fence_before_sync();
     __syncthreads();
+    cluster_sync();   // the barriers of both CTAs are set up
     tc::fence_after_sync();
-    const uint32_t tmem = tmem_slot;
+    const uint32_t tmem = sh.tmem_slot;
+    const uint32_t strip = (uint32_t)px * 128;
+    constexpr int kGroups = 9 / kTaps;
 
-    if (warp == 0) {
-        if (lane == 0) {
-            // loader: slab g of the CTA's sequence uses stage g mod kPStages
-            int g = 0;
-            bool ok = true;
-            for (int tile = blockIdx.x; ok && tile < ntiles; tile += gridDim.x) {
-                const int m0 = tile * 128;
-                const int b = m0 >> (2 * lgS);
-                const int y0 = (m0 >> lgS) & (S - 1), x0 = m0 & (S - 1);
-                for (int s = 0; s < kSlabs; ++s, ++g) {
-                    const int st = g % kPStages;
-                    if (g >= kPStages &&
-                        !tc::mbar_wait_bounded(&empty[st],
-                                               ((g / kPStages) - 1) & 1)) {
-                        atomicOr(&s_fail, 1);
-                        ok = false;
-                        break;
+    if (warp == kEpiWarps) {
+        // strip loader: strip g of the pair's sequence uses stage g mod na
+        const bool leader = elect_one();
+        int g = 0, st = 0;
+        uint32_t ph = 1;   // parity of the stage's last release
+        bool ok = true;
+        for (int pr = pair0; ok && pr < npairs; pr += pstep) {
+            const int m0 = (2 * pr + rank) * 128;
+            const int b = m0 >> (2 * lgS);
+            const int y0 = (m0 >> lgS) & (S - 1), x0 = m0 & (S - 1);
+            for (int q = 0; ok && q < kGroups; ++q) {
+                const int dy = sign * ((kTaps == 3 ? q : q / 3) - 1) * d;
+                const int dx = kTaps == 3 ? -d : sign * (q % 3 - 1) * d;
+                for (int half = 0; half < 2; ++half, ++g) {
+                    if (g >= na) ok = all_ok(tc::mbar_wait_bounded(&sh.aempty[st], ph));
+                    ok = all_ok(ok && !*(volatile int *)&sh.fail);
+                    if (!ok) break;
+                    if (leader) {
+                        if (rank == 0) expect_tx(&sh.afull[st], 2 * strip);
+                        tma_4d_pair(abase + st * strip, &act, half * 64, x0 + dx, y0 + dy,
+                                    b, leader_addr(&sh.afull[st]));
                     }
-                    if (*(volatile int *)&s_fail) {
-                        ok = false;
-                        break;
-                    }
-                    const int tap = s >> 1, c0 = (s & 1) * 64;
-                    const int dy = sign * (tap / 3 - 1) * d;
-                    const int dx = sign * (tap % 3 - 1) * d;
-                    const uint32_t sa = base + st * kStageBytes;
-                    expect_tx(&full[st], kStageBytes);
-                    tma_4d(sa, &act, c0, x0 + dx, y0 + dy, b, &full[st]);
-                    tma_2d(sa + kTileBytes, &wts, s * 64, 0, &full[st]);
+                    __syncwarp();
+                    if (++st == na) st = 0, ph ^= 1;
                 }
             }
-            s_issued = g;
         }
-    } else if (warp == 1) {
-        if (lane == 0) {
-            // MMA issuer: tile number `it` of this CTA accumulates in buffer
-            // it & 1, once the epilogue has drained that buffer's last use
-            constexpr uint32_t idesc = tc::idesc_bf16(128, 128);
-            int g = 0, it = 0;
-            bool ok = true;
-            for (int tile = blockIdx.x; ok && tile < ntiles;
-                 tile += gridDim.x, ++it) {
-                const int acc = it & 1;
-                if (it >= 2 &&
-                    !tc::mbar_wait_bounded(&tempty[acc], ((it >> 1) - 1) & 1)) {
-                    atomicOr(&s_fail, 1);
-                    break;
-                }
-                tc::fence_after_sync();
-                const uint32_t td = tmem + (uint32_t)(acc * 128);
-                for (int s = 0; s < kSlabs; ++s, ++g) {
-                    const int st = g % kPStages;
-                    if (!tc::mbar_wait_bounded(&full[st], (g / kPStages) & 1)) {
-                        atomicOr(&s_fail, 1);
-                        ok = false;
-                        break;
-                    }
-                    tc::fence_after_sync();
-                    const uint32_t sa = base + st * kStageBytes, sb = sa + kTileBytes;
-#pragma unroll
-                    for (int kk = 0; kk < 4; ++kk)
-                        tc::mma_bf16(td, desc_sw128(sa + kk * 32),
-                                     desc_sw128(sb + kk * 32), idesc,
-                                     s > 0 || kk > 0);
-                    tc::mma_commit(&empty[st]);
-                }
-                if (ok) tc::mma_commit(&tfull[acc]);
+        if (leader) {
+            if (!ok) atomicOr(&sh.fail, 1);
+            sh.issued = g;
+        }
+        __syncwarp();
+    } else if (warp == kEpiWarps + 1) {
+        // this CTA's half of the weights: rows 64 rank .. 64 rank + 63
+        const bool leader = elect_one();
+        for (int s = 0; s < kSlabs; ++s) {
+            if (leader) {
+                if (rank == 0) expect_tx(&sh.wfull[s], 2 * kWHalf);
+                tma_2d_pair(wbase + s * kWHalf, &wts, s * 64, 64 * rank,
+                            leader_addr(&sh.wfull[s]));
             }
-            s_consumed = g;
-            tc::mma_commit(&done);   // arrives once every issued MMA is done
+            __syncwarp();
+        }
+    } else if (warp == kEpiWarps + 2) {
+        if (rank == 0) {
+            // MMA issuer: pair number `it` of this cluster accumulates in
+            // buffer it & 1, once the epilogues have drained its last use.
+            // One thread's instruction latency is what an MMA every 64 clocks
+            // competes with, so the waits and commits are per group of taps,
+            // the slabs of a group are unrolled, and the whole warp walks the
+            // loop and votes on its waits, which keeps the operand descriptors
+            // warp-uniform; one elected lane issues.
+            constexpr uint32_t idesc = tc::idesc_bf16(256, 128);
+            const uint64_t adesc = desc_sw128(abase), wdesc = desc_sw128(wbase);
+            const uint32_t strip16 = strip >> 4;
+            // rows of a strip: a tap's shift (a multiple of 128 bytes; the
+            // 128-byte swizzle goes by address, so any row may come first)
+            const uint32_t row0 = sign > 0 ? 0 : (kTaps - 1) * (uint32_t)d * 8;
+            const int rowstep = sign * d * 8;
+            const bool leader = elect_one();
+            int it = 0, ast = 0, ag = 0;
+            uint32_t aph = 0;
+            bool ok = true;
+            for (int pr = pair0; ok && pr < npairs; pr += pstep, ++it) {
+                const int acc = it & 1;
+                if (it >= 2)
+                    ok = all_ok(tc::mbar_wait_bounded(&sh.tempty[acc], ((it >> 1) - 1) & 1));
+                const uint32_t td = tmem + (uint32_t)(acc * 128);
+                for (int q = 0; ok && q < kGroups; ++q) {
+                    // the strips of the two channel halves
+                    const int st0 = ast, st1 = ast + 1 == na ? 0 : ast + 1;
+                    const uint32_t ph1 = ast + 1 == na ? aph ^ 1 : aph;
+                    if (it == 0)
+                        for (int s = 2 * kTaps * q; ok && s < 2 * kTaps * (q + 1); ++s)
+                            ok = all_ok(tc::mbar_wait_bounded(&sh.wfull[s], 0));
+                    ok = ok && all_ok(tc::mbar_wait_bounded(&sh.afull[st0], aph) &&
+                                      tc::mbar_wait_bounded(&sh.afull[st1], ph1));
+                    if (!ok) break;
+                    tc::fence_after_sync();
+                    const uint64_t a0 = adesc + st0 * strip16 + row0;
+                    const uint64_t a1 = adesc + st1 * strip16 + row0;
+                    const uint64_t w0 = wdesc + q * (2 * kTaps * (kWHalf >> 4));
+                    if (leader) {
+#pragma unroll
+                        for (int j = 0; j < kTaps; ++j)
+#pragma unroll
+                            for (int h = 0; h < 2; ++h)
+#pragma unroll
+                                for (int kk = 0; kk < 4; ++kk)
+                                    mma_bf16_pair(
+                                        td, (h ? a1 : a0) + j * rowstep + kk * 2,
+                                        w0 + (2 * j + h) * (kWHalf >> 4) + kk * 2, idesc,
+                                        q > 0 || j > 0 || h > 0 || kk > 0);
+                        commit_pair(&sh.aempty[st0]);
+                        commit_pair(&sh.aempty[st1]);
+                        if (q == kGroups - 1) commit_pair(&sh.tfull[acc]);
+                    }
+                    __syncwarp();
+                    ag += 2;
+                    ast += 2;
+                    if (ast >= na) ast -= na, aph ^= 1;
+                }
+            }
+            if (leader) {
+                if (!ok) atomicOr(&sh.fail, 1);
+                sh.used = ag;
+                commit_pair(&sh.done);   // arrives once every issued MMA is done
+            }
+            __syncwarp();
         }
     } else {
-        // epilogue: tile number `it` is read from buffer it & 1
-        const int q = warp & 3;   // tensor-memory lane quarter of this warp
+        // epilogue: pair number `it` is read from buffer it & 1
         int it = 0;
-        for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++it) {
+        for (int pr = pair0; pr < npairs; pr += pstep, ++it) {
             const int acc = it & 1;
-            if (*(volatile int *)&s_fail) break;
-            if (!tc::mbar_wait_bounded(&tfull[acc], (it >> 1) & 1)) {
-                atomicOr(&s_fail, 1);
+            const size_t p = (size_t)(2 * pr + rank) * 128 + warp * 32 + lane;
+            uint32_t mask[64];
+            if (epi.mode != 0) {
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    ld_global32(epi.hprev + p * 128 + 16 * j, mask + 8 * j);
+            }
+            if (*(volatile int *)&sh.fail ||
+                !tc::mbar_wait_bounded(&sh.tfull[acc], (it >> 1) & 1)) {
+                atomicOr(&sh.fail, 1);
                 break;
             }
             tc::fence_after_sync();
-            conv_epilogue(epi, s_bias,
-                          tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * 128),
-                          tile * 128 + q * 32 + lane);
+            pair_epilogue(epi, sh.bias,
+                          tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(acc * 128), p,
+                          mask);
             tc::fence_before_sync();
-            mbar_arrive(&tempty[acc]);
+            __syncwarp();
+            if (lane == 0) arrive_cluster(leader_addr(&sh.tempty[acc]));
         }
     }
     __syncthreads();
     if (tid == 0) {
-        if (s_fail) {
+        if (sh.fail) {
             atomicOr(err, 1u);
-            // copies issued but never consumed must land before the CTA leaves
-            for (int g = s_consumed; g < s_issued; ++g)
-                tc::mbar_wait_bounded(&full[g % kPStages], (g / kPStages) & 1);
+            // copies of either CTA still in flight must land before the pair
+            // leaves: the leader waits for those it can see (bounded), both
+            // for a time far above a copy's
+            if (rank == 0)
+                for (int g = sh.used; g < sh.issued; ++g)
+                    tc::mbar_wait_bounded(&sh.afull[g % na], (g / na) & 1);
+            const long long t0 = clock64();
+            while (clock64() - t0 < (1ll << 24)) {}
         }
-        // every MMA this CTA issued has completed
-        tc::mbar_wait_bounded(&done, 0);
+        // every MMA of the pair has completed
+        tc::mbar_wait_bounded(&sh.done, 0);
     }
     tc::fence_before_sync();
     __syncthreads();
+    cluster_sync();   // neither CTA leaves while the other may signal it
     tc::fence_after_sync();
-    if (warp == 0) tc::tmem_dealloc(tmem, 256);
+    if (warp == kEpiWarps) tmem_dealloc_pair(tmem, 256);
 }
 
 // Weight gradient of a 128 -> 128 layer: D[o][(t, i)] = sum_p dz[p, o]
@@ -695,13 +785,24 @@ bool map_act(CUtensorMap *m, const uint16_t *ptr, int n, int S, int pix = 128)
     if (!fn) return false;
     const cuuint64_t dims[4] = {128, (cuuint64_t)S, (cuuint64_t)S, (cuuint64_t)n};
     const cuuint64_t strides[3] = {256, (cuuint64_t)S * 256, (cuuint64_t)S * S * 256};
-    const cuuint32_t bx = S >= pix ? pix : S, by = pix / bx;
+    const cuuint32_t bx = S >= 128 || S >= pix ? pix : S, by = pix / bx;
     const cuuint32_t box[4] = {64, bx, by, 1};
     const cuuint32_t es[4] = {1, 1, 1, 1};
     return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<uint16_t *>(ptr), dims,
               strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
               CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// Strips of the pair convolution.  Three taps share a strip when a CTA's 128
+// pixels lie in one row (S >= 128) and three strips fit in shared memory (two
+// serve a row of taps, one is filled meanwhile): dilations up to 32.
+StripShape conv_shape(int S, int d)
+{
+    StripShape sp{3, 128 + (2 * d + 7) / 8 * 8, 0};
+    if (S < 128 || 3 * sp.px * 128 > kStripRoom) sp = StripShape{1, 128, 0};
+    sp.na = std::min(kMaxA, kStripRoom / (sp.px * 128));
+    return sp;
 }
 
 // First-layer input [n][S][S][16] BF16; box 16 channels x 128 pixels.
@@ -735,14 +836,14 @@ bool map_w144(CUtensorMap *m, const uint16_t *ptr)
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// Weights [128 rows][1152] BF16; box 64 x 128.
+// Weights [128 rows][1152] BF16; box 64 x 64 (one CTA's half of a slab).
 bool map_wts(CUtensorMap *m, const uint16_t *ptr)
 {
     auto fn = encoder();
     if (!fn) return false;
     const cuuint64_t dims[2] = {1152, 128};
     const cuuint64_t strides[1] = {1152 * 2};
-    const cuuint32_t box[2] = {64, 128};
+    const cuuint32_t box[2] = {64, 64};
     const cuuint32_t es[2] = {1, 1};
     return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<uint16_t *>(ptr), dims,
               strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
@@ -764,30 +865,23 @@ cudaError_t launch_conv_tma(int mode, const uint16_t *in, const uint16_t *w,
     using namespace convtma;
     if (S < 16 || (S & (S - 1)) || ((uintptr_t)in & 15) || ((uintptr_t)w & 15))
         return cudaErrorInvalidValue;
+    const StripShape sp = conv_shape(S, d);
     CUtensorMap ma, mw;
-    if (!map_act(&ma, in, n, S) || !map_wts(&mw, w)) return cudaErrorInvalidValue;
+    if (!map_act(&ma, in, n, S, sp.px) || !map_wts(&mw, w)) return cudaErrorInvalidValue;
     Epi e{mode, bias, hprev, out};
-    const long long P = (long long)n * S * S;
-    const int ntiles = (int)(P / 128);
-#if FIRE_CONV_PERSISTENT
     int dev = 0, nsm = 0;
     cudaError_t attr = cudaGetDevice(&dev);
     if (attr == cudaSuccess)
         attr = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    const auto kern = sp.taps == 3 ? k_conv_pair<3> : k_conv_pair<1>;
     if (attr == cudaSuccess)
-        attr = cudaFuncSetAttribute(k_conv_tma_p,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize, kPSmem);
+        attr = cudaFuncSetAttribute(
+            kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kPairSmem);
     if (attr != cudaSuccess) return attr;
-    const int grid = std::min(ntiles, 2 * nsm);
-    k_conv_tma_p<<<grid, kPThreads, kPSmem, st>>>(ma, mw, e, S, lgS, d,
-                                                  mode == 0 ? 1 : -1, ntiles, err);
-#else
-    cudaError_t attr = cudaFuncSetAttribute(
-        k_conv_tma, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
-    if (attr != cudaSuccess) return attr;
-    k_conv_tma<<<(unsigned)ntiles, 128, kSmem, st>>>(ma, mw, e, S, lgS, d,
-                                                     mode == 0 ? 1 : -1, err);
-#endif
+    // S >= 16: whole pairs of 128-pixel tiles
+    const int npairs = (int)((long long)n * S * S / 256);
+    kern<<<2 * std::min(npairs, nsm / 2), kPairThreads, kPairSmem, st>>>(
+        ma, mw, e, sp.px, sp.na, S, lgS, d, mode == 0 ? 1 : -1, npairs, err);
     return cudaGetLastError();
 }
 

@@ -129,6 +129,7 @@ __device__ __forceinline__ bool mbar_try_wait(void *bar, uint32_t parity)
 // Bounded wait (about a second of clocks); false when it ran out.
 __device__ __forceinline__ bool mbar_wait_bounded(void *bar, uint32_t parity)
 {
+    if (mbar_try_wait(bar, parity)) return true;   // the clock only when it must wait
     const long long t0 = clock64();
     while (!mbar_try_wait(bar, parity)) {
         if (clock64() - t0 > (1ll << 31)) return false;
