@@ -307,6 +307,7 @@ int fire_maps_upload(fire_ctx *ctx, int H, int W, float cell_m,
         (e = cudaMalloc(&m->ps, HW * sizeof(float2))) != cudaSuccess ||
         (e = cudaMalloc(&m->cfl, HW * sizeof(uint16_t))) != cudaSuccess ||
         (e = cudaMalloc(&m->blk, words * 4)) != cudaSuccess ||
+        (e = cudaMalloc(&m->init, words * 8)) != cudaSuccess ||
         (e = cudaMalloc(&m->tgt, words * 4)) != cudaSuccess ||
         (e = cudaMalloc(&m->tgt_count, 16)) != cudaSuccess) {
         fire_map_free(m);
@@ -318,6 +319,7 @@ int fire_maps_upload(fire_ctx *ctx, int H, int W, float cell_m,
     m->dev.ps = m->ps;
     m->dev.cfl = m->cfl;
     m->dev.blk = m->blk;
+    m->dev.init = m->init;
     m->dev.tgt = m->tgt;
     m->dev.tgt_count = m->tgt_count;
 
@@ -376,7 +378,7 @@ int fire_maps_upload(fire_ctx *ctx, int H, int W, float cell_m,
         m->dev.om1 = w0.x;
         m->dev.om3 = w0.y;
     }
-    if (e == cudaSuccess) e = launch_blocked(m->dev, dveg, m->blk, ctx->stream);
+    if (e == cudaSuccess) e = launch_blocked(m->dev, dveg, m->blk, m->init, ctx->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(m->tgt, 0, words * 4, ctx->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(m->tgt_count, 0, 16, ctx->stream);
     // host copy of the burnable mask for validating host ignitions
@@ -408,6 +410,7 @@ void fire_map_free(fire_map *m)
     if (m->ps) cudaFree(m->ps);
     if (m->cfl) cudaFree(m->cfl);
     if (m->blk) cudaFree(m->blk);
+    if (m->init) cudaFree(m->init);
     if (m->tgt) cudaFree(m->tgt);
     if (m->tgt_count) cudaFree(m->tgt_count);
     delete m;

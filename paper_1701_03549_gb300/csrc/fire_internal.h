@@ -32,6 +32,8 @@ struct MapDev {
     float cw, sw, om1, om3;
     const uint16_t *cfl;        // bit d<8 uphill from source d, 8 forest, 9 burnable
     const uint32_t *blk;        // non-burnable bitmap, ntiles * 32 words
+    const uint2 *init;          // every word of blk twice: a simulation's initial
+                                // state (X, Y), ntiles * 32 pairs
     const uint32_t *tgt;        // target bitmap, ntiles * 32 words
     const uint32_t *tgt_count;  // |A|, one word
 };
@@ -54,7 +56,7 @@ struct SimLaunch {
                                // cleared), ntiles * 32 words per simulation
     uint32_t *work_counter;    // zeroed before launch
     uint32_t *gstate;          // global-state variant: block_words words per block
-    size_t block_words;        // 0: 2 * ntiles_max * 32 (the X, Y planes)
+    size_t block_words;        // 0: 2 * ntiles_max * 32 (the (X, Y) pairs)
     const uint8_t *burn_time;  // burn-time variant: steps each cell burns
                                // (1..250, others clamped); its blocks keep X, Y,
                                // two "still burning" planes and one fuel byte
@@ -102,7 +104,7 @@ struct SimShared {
 // Shared-memory layout of the simulation kernel (identical on host/device):
 // header, worklist mark bits (2 per tile), three worklists of uint16 tile
 // indices, the block's candidate queue (qcap uint32 entries), then, in the
-// shared-state variant, the X and Y planes.
+// shared-state variant, the (X, Y) state pairs.
 struct SimLayout {
     size_t header, marks, lists, queue, planes, total;
 };
@@ -132,7 +134,7 @@ cudaError_t launch_features(int H, int W, const uint8_t *veg, const float *elev,
                             float2 *ps, uint16_t *cfl, uint32_t *wind_varies,
                             cudaStream_t st);
 cudaError_t launch_blocked(const MapDev &m, const uint8_t *veg, uint32_t *blk,
-                           cudaStream_t st);
+                           uint2 *init, cudaStream_t st);
 cudaError_t launch_target(const MapDev &m, const uint8_t *burnt, uint32_t *tgt,
                           uint32_t *tgt_count, cudaStream_t st);
 cudaError_t launch_simulate(const SimLaunch &a, bool smem_state, int nwarps,
@@ -240,6 +242,7 @@ struct fire_map {
     float2 *ps = nullptr;
     uint16_t *cfl = nullptr;
     uint32_t *blk = nullptr;
+    uint2 *init = nullptr;
     uint32_t *tgt = nullptr;
     uint32_t *tgt_count = nullptr;
     std::vector<uint8_t> burnable_host;

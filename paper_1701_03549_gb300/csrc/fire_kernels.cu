@@ -102,6 +102,7 @@ template <bool kTarget>
 __global__ void k_pack_bits(int H, int W, int TW, int nwords,
                             const uint8_t *__restrict__ src,
                             uint32_t *__restrict__ dst,
+                            uint2 *__restrict__ init,
                             uint32_t *__restrict__ count)
 {
     const int w = blockIdx.x * blockDim.x + threadIdx.x;
@@ -119,6 +120,7 @@ __global__ void k_pack_bits(int H, int W, int TW, int nwords,
             word |= (uint32_t)bit << i;
         }
         dst[w] = word;
+        if (!kTarget) init[w] = make_uint2(word, word);
     }
     if (kTarget) {
         uint32_t c = __reduce_add_sync(kFull, w < nwords ? __popc(word) : 0u);
@@ -201,10 +203,11 @@ __device__ __forceinline__ void fence_proxy_async_smem()
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
 
-__device__ __forceinline__ uint32_t burning(uint32_t x, uint32_t y,
-                                            uint32_t par)
+// Cells of a state pair that burn at a step whose parity mask pm is 0 (even)
+// or ~0 (odd): code 10 or 01.  One three-input logic operation.
+__device__ __forceinline__ uint32_t burning(uint2 s, uint32_t pm)
 {
-    return par ? (y & ~x) : (x & ~y);
+    return (s.x & ~s.y & ~pm) | (~s.x & s.y & pm);
 }
 
 struct SimCtx {
@@ -214,7 +217,7 @@ struct SimCtx {
     uint32_t *marks;
     uint16_t *lists;
     uint32_t *queue;
-    uint32_t *X, *Y;
+    uint2 *P;            // state pairs (X, Y), one per row word
     uint32_t *K0, *K1;   // burn-time variant: cells still burning, by step parity
     uint8_t *fuel;       // burn-time variant: steps of fuel left per cell
     int ntiles;
@@ -361,8 +364,9 @@ __device__ __forceinline__ void ignite(const SimCtx &s, int k, int ti, int tj,
                                        int r, int i, uint32_t cell, uint32_t t)
 {
     const MapDev &m = *s.map;
-    uint32_t *P = (t & 1u) ? s.X : s.Y;
-    atomicOr(&P[k * 32 + r], 1u << i);
+    // burning at odd steps is code 01 (Y), at even steps 10 (X)
+    uint32_t *word = reinterpret_cast<uint32_t *>(&s.P[k * 32 + r]) + ((t & 1u) ^ 1u);
+    atomicOr(word, 1u << i);
     if (kBurn) {
         // only cells that burn two steps or more keep a fuel count
         const uint8_t f = burn_steps(*s.a, cell);
@@ -397,6 +401,19 @@ __device__ __forceinline__ int nth_set_bit(uint32_t m, uint32_t n)
     return pos;
 }
 
+// Directions with a burning source from the three-column windows (bit 0 the
+// left column) of the rows above, at and below a target.  The source of
+// direction d lies at target - off(d): N below, NE below left, E left, SE
+// above left, S above, SW above right, W right, NW below right.
+__device__ __forceinline__ uint32_t dir_mask(uint32_t up, uint32_t mid, uint32_t down)
+{
+    // tables of eight bytes indexed by a window: its bits moved to
+    // E (2), W (6) and to NE (1), N (0), NW (7)
+    const uint32_t m = __byte_perm(0x04000400u, 0x44404440u, mid);
+    const uint32_t d = __byte_perm(0x03010200u, 0x83818280u, down);
+    return (up << 3) | m | d;
+}
+
 // Phase A of step t for active tile k, one warp (lane = tile row): retire the
 // previous step's burning cells, find the targets with a burning source in
 // each direction, count the trials and queue the candidates for phase B.
@@ -409,26 +426,28 @@ __device__ __forceinline__ void phase_a(const SimCtx &s, int k, uint32_t t,
     SimShared &sh = *s.sh;
     const int TW = m.TW, TH = m.TH;
     const int ti = tile_row(sh, k), tj = k - ti * TW;
-    const uint32_t par = t & 1u;
-    uint32_t *X = s.X, *Y = s.Y;
+    const uint32_t par = t & 1u, pm = 0u - par;
     // burn-time variant: the sources of step t also include the cells that
     // ignited before step t - 1 and still burn (plane K[t & 1])
     const uint32_t *Kt = kBurn ? (par ? s.K1 : s.K0) : nullptr;
 
     if (lane == 0) atomicAnd(&s.marks[k >> 4], ~(1u << (2 * (k & 15) + par)));
 
+    // Sources of this row (b) and the two beyond its ends (ext: bit 0 left,
+    // bit 1 right).
     const int w = k * 32 + lane;
-    const uint32_t x = X[w], y = Y[w];
-    uint32_t b = burning(x, y, par);
+    const uint2 own = s.P[w];
+    uint32_t b = burning(own, pm), ext = 0;
     if (kBurn) b |= Kt[w];
-    uint32_t bl = 0, br = 0;
     if (tj > 0) {
-        bl = burning(X[w - 32], Y[w - 32], par);
-        if (kBurn) bl |= Kt[w - 32];
+        uint32_t l = burning(s.P[w - 32], pm);
+        if (kBurn) l |= Kt[w - 32];
+        ext = l >> 31;
     }
     if (tj < TW - 1) {
-        br = burning(X[w + 32], Y[w + 32], par);
-        if (kBurn) br |= Kt[w + 32];
+        uint32_t r = burning(s.P[w + 32], pm);
+        if (kBurn) r |= Kt[w + 32];
+        ext |= (r & 1u) << 1;
     }
     // Edge rows of the tiles above (row 31) and below (row 0), including the
     // diagonal neighbours: lanes 0..5 fetch one word each.
@@ -439,39 +458,31 @@ __device__ __forceinline__ void phase_a(const SimCtx &s, int k, uint32_t t,
         const int nti = ti + dti, ntj = tj + dtj;
         if (nti >= 0 && nti < TH && ntj >= 0 && ntj < TW) {
             const int we = (nti * TW + ntj) * 32 + (dti < 0 ? 31 : 0);
-            edge = burning(X[we], Y[we], par);
+            edge = burning(s.P[we], pm);
             if (kBurn) edge |= Kt[we];
         }
     }
-    uint32_t bu = __shfl_up_sync(kFull, b, 1);
-    uint32_t blu = __shfl_up_sync(kFull, bl, 1);
-    uint32_t bru = __shfl_up_sync(kFull, br, 1);
-    uint32_t bd = __shfl_down_sync(kFull, b, 1);
-    uint32_t bld = __shfl_down_sync(kFull, bl, 1);
-    uint32_t brd = __shfl_down_sync(kFull, br, 1);
-    const uint32_t e_ul = __shfl_sync(kFull, edge, 0);
+    // The rows above (bu) and below (bd) with their ends.  Of a diagonal
+    // neighbour only one bit counts: bit 31 on the left (lanes 0, 3), bit 0
+    // on the right (lanes 2, 5).
+    const uint32_t diag =
+        __ballot_sync(kFull, (lane == 0 || lane == 3 ? edge >> 31 : edge & 1u) != 0);
     const uint32_t e_u = __shfl_sync(kFull, edge, 1);
-    const uint32_t e_ur = __shfl_sync(kFull, edge, 2);
-    const uint32_t e_dl = __shfl_sync(kFull, edge, 3);
     const uint32_t e_d = __shfl_sync(kFull, edge, 4);
-    const uint32_t e_dr = __shfl_sync(kFull, edge, 5);
+    uint32_t bu = __shfl_up_sync(kFull, b, 1), xu = __shfl_up_sync(kFull, ext, 1);
+    uint32_t bd = __shfl_down_sync(kFull, b, 1), xd = __shfl_down_sync(kFull, ext, 1);
     if (lane == 0) {
         bu = e_u;
-        blu = e_ul;
-        bru = e_ur;
+        xu = (diag & 1u) | ((diag >> 1) & 2u);
     }
     if (lane == 31) {
         bd = e_d;
-        bld = e_dl;
-        brd = e_dr;
+        xd = ((diag >> 3) & 1u) | ((diag >> 4) & 2u);
     }
     // Retire last step's burning cells (code of parity t + 1) to "burnt";
     // readers of other tiles only look for the parity-t code.
-    const uint32_t stale = burning(x, y, par ^ 1u);
-    if (stale) {
-        X[w] = x | stale;
-        Y[w] = y | stale;
-    }
+    const uint32_t stale = burning(own, ~pm);
+    if (stale) s.P[w] = make_uint2(own.x | stale, own.y | stale);
     if (kBurn) {
         // each cell burning at step t spends one step of fuel; the ones left
         // with fuel burn at step t + 1 as well (plane K[(t + 1) & 1], written
@@ -510,24 +521,17 @@ __device__ __forceinline__ void phase_a(const SimCtx &s, int k, uint32_t t,
     if (__any_sync(kFull, b != 0) && lane == 0) mark_tile(s, k, t + 1);
     __syncwarp();
 
-    // Targets of row `lane` with a burning source in direction d (the source
-    // of direction d lies at target - off(d)).
-    const uint32_t avail = ~(x | y);
-    uint32_t md[8];
-    md[0] = bd;                               // N : source below
-    md[1] = (bd << 1) | (bld >> 31);          // NE: source below-left
-    md[2] = (b << 1) | (bl >> 31);            // E : source left
-    md[3] = (bu << 1) | (blu >> 31);          // SE: source above-left
-    md[4] = bu;                               // S : source above
-    md[5] = (bu >> 1) | (bru << 31);          // SW: source above-right
-    md[6] = (b >> 1) | (br << 31);            // W : source right
-    md[7] = (bd >> 1) | (brd << 31);          // NW: source below-right
-    uint32_t cand = 0;
-#pragma unroll
-    for (int d = 0; d < 8; ++d) {
-        md[d] &= avail;
-        cand |= md[d];
-    }
+    // Candidates: available cells with a source in the 3 x 3 window around
+    // them (an available cell is no source itself).
+    const uint32_t v = bu | b | bd, xv = xu | ext | xd;
+    const uint32_t cand = ~(own.x | own.y) &
+                          (v | ((v << 1) | (xv & 1u)) | __funnelshift_r(v, xv >> 1, 1));
+    // Each row's sources shifted left by one, with the left end in bit 0; the
+    // two bits above (bit 31 and the right end) of all three rows packed.
+    const uint32_t lu = (bu << 1) | (xu & 1u), lc = (b << 1) | (ext & 1u),
+                   ld = (bd << 1) | (xd & 1u);
+    const uint32_t hi3 = ((bu >> 31) | (xu & 2u)) | (((b >> 31) | (ext & 2u)) << 2) |
+                         (((bd >> 31) | (xd & 2u)) << 4);
     const uint32_t c = __popc(cand);
     uint32_t incl = c;
 #pragma unroll
@@ -563,10 +567,12 @@ __device__ __forceinline__ void phase_a(const SimCtx &s, int k, uint32_t t,
         const uint32_t cr = __shfl_sync(kFull, cand, r);
         const uint32_t ir = __shfl_sync(kFull, incl, r);
         const int i = nth_set_bit(cr, q - (ir - (uint32_t)__popc(cr)));
-        uint32_t dm = 0;
-#pragma unroll
-        for (int d = 0; d < 8; ++d)
-            dm |= ((__shfl_sync(kFull, md[d], r) >> i) & 1u) << d;
+        // the columns i - 1, i, i + 1 of the rows above, at and below
+        const uint32_t h3 = __shfl_sync(kFull, hi3, r);
+        const uint32_t wu = __funnelshift_r(__shfl_sync(kFull, lu, r), h3, i);
+        const uint32_t wc = __funnelshift_r(__shfl_sync(kFull, lc, r), h3 >> 2, i);
+        const uint32_t wd = __funnelshift_r(__shfl_sync(kFull, ld, r), h3 >> 4, i);
+        const uint32_t dm = dir_mask(wu & 7u, wc & 7u, wd & 7u);
         if (q >= total) continue;
         if (base != 0xffffffffu) {
             s.queue[base + q] = ((uint32_t)(k * 32 + r) << 13) |
@@ -604,17 +610,16 @@ __global__ void __launch_bounds__(kSimMaxThreads, 2) k_simulate(SimLaunch a)
     s.queue = reinterpret_cast<uint32_t *>(smem + L.queue);
     s.ntiles = ntiles_max;
     if (kSmemState) {
-        s.X = reinterpret_cast<uint32_t *>(smem + L.planes);
+        s.P = reinterpret_cast<uint2 *>(smem + L.planes);
     } else {
         const size_t stride =
             a.block_words ? a.block_words : 2 * (size_t)ntiles_max * 32;
-        s.X = a.gstate + (size_t)blockIdx.x * stride;
+        s.P = reinterpret_cast<uint2 *>(a.gstate + (size_t)blockIdx.x * stride);
     }
-    s.Y = s.X + ntiles_max * 32;
     s.K0 = s.K1 = nullptr;
     s.fuel = nullptr;
     if (kBurn) {
-        s.K0 = s.Y + ntiles_max * 32;
+        s.K0 = reinterpret_cast<uint32_t *>(s.P + ntiles_max * 32);
         s.K1 = s.K0 + ntiles_max * 32;
         s.fuel = reinterpret_cast<uint8_t *>(s.K1 + ntiles_max * 32);
     }
@@ -680,32 +685,30 @@ __global__ void __launch_bounds__(kSimMaxThreads, 2) k_simulate(SimLaunch a)
             sh.inter = 0;
         }
         __syncthreads();   // the map descriptor is read by every thread below
-        const uint32_t plane_bytes = (uint32_t)m.ntiles * 128u;
+        const uint32_t state_bytes = (uint32_t)m.ntiles * 256u;
         const long long HW = (long long)m.H * m.W;
         for (int i = threadIdx.x; i < sh.nmark; i += blockDim.x) s.marks[i] = 0;
         if (kSmemState) {
             fence_proxy_async_smem();
             __syncthreads();
             if (threadIdx.x == 0) {
-                mbar_arrive_expect_tx(&sh.mbar, 2u * plane_bytes);
-                bulk_g2s(s.X, m.blk, plane_bytes, &sh.mbar);
-                bulk_g2s(s.Y, m.blk, plane_bytes, &sh.mbar);
+                mbar_arrive_expect_tx(&sh.mbar, state_bytes);
+                bulk_g2s(s.P, m.init, state_bytes, &sh.mbar);
             }
         } else {
             const uint4 *src = reinterpret_cast<const uint4 *>(m.blk);
-            uint4 *dx = reinterpret_cast<uint4 *>(s.X);
-            uint4 *dy = reinterpret_cast<uint4 *>(s.Y);
+            uint4 *dst = reinterpret_cast<uint4 *>(s.P);
             // two 16-byte loads in flight per thread before their stores
             const int n16 = m.ntiles * 8, bd = blockDim.x;
             for (int i = threadIdx.x; i < n16; i += 2 * bd) {
                 const bool two = i + bd < n16;
                 const uint4 v0 = src[i];
                 const uint4 v1 = two ? src[i + bd] : v0;
-                dx[i] = v0;
-                dy[i] = v0;
+                dst[2 * i] = make_uint4(v0.x, v0.x, v0.y, v0.y);
+                dst[2 * i + 1] = make_uint4(v0.z, v0.z, v0.w, v0.w);
                 if (two) {
-                    dx[i + bd] = v1;
-                    dy[i + bd] = v1;
+                    dst[2 * (i + bd)] = make_uint4(v1.x, v1.x, v1.y, v1.y);
+                    dst[2 * (i + bd) + 1] = make_uint4(v1.z, v1.z, v1.w, v1.w);
                 }
             }
             if (kBurn) {
@@ -751,7 +754,7 @@ __global__ void __launch_bounds__(kSimMaxThreads, 2) k_simulate(SimLaunch a)
             } else {
                 const int k0 = (g.row >> 5) * m.TW + (g.col >> 5);
                 const int r0 = g.row & 31, i0 = g.col & 31;
-                s.X[k0 * 32 + r0] |= 1u << i0;   // burning, parity 0
+                s.P[k0 * 32 + r0].x |= 1u << i0;   // burning, parity 0
                 if (kBurn) {
                     const uint32_t c0 = (uint32_t)g.row * (uint32_t)m.W + (uint32_t)g.col;
                     const uint8_t f = burn_steps(a, c0);
@@ -837,7 +840,7 @@ __global__ void __launch_bounds__(kSimMaxThreads, 2) k_simulate(SimLaunch a)
         bool border = false;
         if (a.burnt_bits) {
             for (int w = threadIdx.x; w < m.ntiles * 32; w += blockDim.x) {
-                const uint32_t bw = (s.X[w] | s.Y[w]) & ~__ldg(&m.blk[w]);
+                const uint32_t bw = (s.P[w].x | s.P[w].y) & ~__ldg(&m.blk[w]);
                 a.burnt_bits[(long long)sim * m.ntiles * 32 + w] = bw;
                 if (!bw) continue;
                 nb += __popc(bw);
@@ -851,14 +854,13 @@ __global__ void __launch_bounds__(kSimMaxThreads, 2) k_simulate(SimLaunch a)
             }
         } else {
             // four consecutive rows of one tile per thread (16-byte loads)
-            const uint4 *X4 = reinterpret_cast<const uint4 *>(s.X);
-            const uint4 *Y4 = reinterpret_cast<const uint4 *>(s.Y);
+            const uint4 *P4 = reinterpret_cast<const uint4 *>(s.P);
             const uint4 *B4 = reinterpret_cast<const uint4 *>(m.blk);
             const uint4 *T4 = reinterpret_cast<const uint4 *>(m.tgt);
             for (int v = threadIdx.x; v < m.ntiles * 8; v += blockDim.x) {
-                const uint4 x = X4[v], y = Y4[v], bl = __ldg(&B4[v]);
-                const uint32_t bw[4] = {(x.x | y.x) & ~bl.x, (x.y | y.y) & ~bl.y,
-                                        (x.z | y.z) & ~bl.z, (x.w | y.w) & ~bl.w};
+                const uint4 p = P4[2 * v], q = P4[2 * v + 1], bl = __ldg(&B4[v]);
+                const uint32_t bw[4] = {(p.x | p.y) & ~bl.x, (p.z | p.w) & ~bl.y,
+                                        (q.x | q.y) & ~bl.z, (q.z | q.w) & ~bl.w};
                 if (!(bw[0] | bw[1] | bw[2] | bw[3])) continue;
                 const uint4 tg = __ldg(&T4[v]);
                 nb += __popc(bw[0]) + __popc(bw[1]) + __popc(bw[2]) + __popc(bw[3]);
@@ -1203,11 +1205,11 @@ cudaError_t launch_features(int H, int W, const uint8_t *veg, const float *elev,
 }
 
 cudaError_t launch_blocked(const MapDev &m, const uint8_t *veg, uint32_t *blk,
-                           cudaStream_t st)
+                           uint2 *init, cudaStream_t st)
 {
     const int nw = m.ntiles * 32;
     k_pack_bits<false><<<(nw + 255) / 256, 256, 0, st>>>(m.H, m.W, m.TW, nw,
-                                                         veg, blk, nullptr);
+                                                         veg, blk, init, nullptr);
     return cudaGetLastError();
 }
 
@@ -1218,7 +1220,8 @@ cudaError_t launch_target(const MapDev &m, const uint8_t *burnt, uint32_t *tgt,
     cudaError_t e = cudaMemsetAsync(tgt_count, 0, sizeof(uint32_t), st);
     if (e != cudaSuccess) return e;
     k_pack_bits<true><<<(nw + 255) / 256, 256, 0, st>>>(m.H, m.W, m.TW, nw,
-                                                        burnt, tgt, tgt_count);
+                                                        burnt, tgt, nullptr,
+                                                        tgt_count);
     return cudaGetLastError();
 }
 
