@@ -304,7 +304,6 @@ int fire_maps_upload(fire_ctx *ctx, int H, int W, float cell_m,
     cudaError_t e = cudaSuccess;
     if ((e = cudaMalloc(&m->feat, HW * sizeof(float4))) != cudaSuccess ||
         (e = cudaMalloc(&m->wdiag, HW * sizeof(float2))) != cudaSuccess ||
-        (e = cudaMalloc(&m->ps, HW * sizeof(float2))) != cudaSuccess ||
         (e = cudaMalloc(&m->cfl, HW * sizeof(uint16_t))) != cudaSuccess ||
         (e = cudaMalloc(&m->blk, words * 4)) != cudaSuccess ||
         (e = cudaMalloc(&m->init, words * 8)) != cudaSuccess ||
@@ -316,7 +315,6 @@ int fire_maps_upload(fire_ctx *ctx, int H, int W, float cell_m,
     }
     m->dev.feat = m->feat;
     m->dev.wdiag = m->wdiag;
-    m->dev.ps = m->ps;
     m->dev.cfl = m->cfl;
     m->dev.blk = m->blk;
     m->dev.init = m->init;
@@ -354,29 +352,36 @@ int fire_maps_upload(fire_ctx *ctx, int H, int W, float cell_m,
         daspect = f[2];
         dwind = f[3];
     }
-    // the map's tgt_count word doubles as the wind-uniformity flag until the
-    // target is cleared below
+    // the map's tgt_count words carry the covariates' flags (the wind varies, a
+    // cell is out of the fixed-point range) until the target is cleared below
     e = launch_features(H, W, dveg, delev, dslope, daspect, dwind, m->feat,
-                        m->wdiag, m->ps, m->cfl, m->tgt_count, ctx->stream);
-    uint32_t wind_varies = 1;
+                        m->wdiag, m->cfl, m->tgt_count, ctx->stream);
+    uint32_t fl[2] = {1, 1};
     float4 f0;
-    float2 w0;
     if (e == cudaSuccess)
-        e = cudaMemcpyAsync(&wind_varies, m->tgt_count, 4, cudaMemcpyDeviceToHost,
+        e = cudaMemcpyAsync(fl, m->tgt_count, sizeof fl, cudaMemcpyDeviceToHost,
                             ctx->stream);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(&f0, m->feat, sizeof f0, cudaMemcpyDeviceToHost,
                             ctx->stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(&w0, m->wdiag, sizeof w0, cudaMemcpyDeviceToHost,
-                            ctx->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
-    if (e == cudaSuccess && !wind_varies) {
-        m->dev.uniform_wind = 1;
-        m->dev.cw = f0.z;
-        m->dev.sw = f0.w;
-        m->dev.om1 = w0.x;
-        m->dev.om3 = w0.y;
+    if (e == cudaSuccess && !fl[1]) {
+        m->dev.fx = 1;
+        m->dev.uniform_wind = !fl[0];
+        m->dev.cw = (int)std::lrintf(f0.z * kFxOne);
+        m->dev.sw = (int)std::lrintf(f0.w * kFxOne);
+        e = cudaMalloc(&m->fx, HW * (fl[0] ? sizeof(int4) : sizeof(int2)));
+        if (e == cudaSuccess) {
+            m->dev.fx2 = fl[0] ? nullptr : (const int2 *)m->fx;
+            m->dev.fx4 = fl[0] ? (const int4 *)m->fx : nullptr;
+            e = launch_fx((long long)HW, m->feat, (int2 *)m->dev.fx2, (int4 *)m->dev.fx4,
+                          ctx->stream);
+        } else {
+            if (tmp) cudaFree(tmp);
+            fire_map_free(m);
+            return set_err(ctx, FIRE_ENOMEM, "map allocation: %s",
+                           cudaGetErrorString(e));
+        }
     }
     if (e == cudaSuccess) e = launch_blocked(m->dev, dveg, m->blk, m->init, ctx->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(m->tgt, 0, words * 4, ctx->stream);
@@ -407,7 +412,7 @@ void fire_map_free(fire_map *m)
     if (m->ctx) cudaSetDevice(m->ctx->device);
     if (m->feat) cudaFree(m->feat);
     if (m->wdiag) cudaFree(m->wdiag);
-    if (m->ps) cudaFree(m->ps);
+    if (m->fx) cudaFree(m->fx);
     if (m->cfl) cudaFree(m->cfl);
     if (m->blk) cudaFree(m->blk);
     if (m->init) cudaFree(m->init);

@@ -383,6 +383,100 @@ __device__ __forceinline__ float screen_p(float z)
     return r;
 }
 
+// ---------------------------------------------------------------------------
+// Fixed-point screen: the same z as a sum of 32 x 32 -> 64 bit products, one
+// multiply-add instruction per term of Eq. 1 (the float pairs above take about
+// twelve operations per term, and a trial's instruction chain is what the
+// simulation kernel spends its time on).  Features are integers of scale 2^30
+// (psi, sig, cos and sin of the wind bearing: |x| <= 1, |sig| < 2),
+// coefficients of scale 2^(k+2), sums of scale 2^(k+32); z is the sum's high
+// word, scale 2^k.  The diagonal wind terms are b3 / sqrt(2) times cos and sin
+// each, so no diagonal cosine is read.  k is 23, or 22 for larger
+// coefficients, so that no coefficient and no sum overflows.
+//
+// Error in z: coefficients rounded to 2^-(k+3), 4.5 of them at most (|psi| 1,
+// wind 1.42, |sig| 2); features rounded to 2^-31 times at most 3.5 max|b|,
+// with max|b| < 2^(29-k); the high word to 2^-(k+1): for k = 22 below 1.4e-7 +
+// 2.1e-7 + 1.2e-7 = 4.7e-7, for k = 23 below 2.4e-7.  z's conversion to float
+// is exact up to 2^24 and 2^-24 relative above, as in the float-pair screen.
+// So p is within 1.2e-7 (6e-8) of z's share and 3.1e-7 + 0.23 2^-24 of the
+// exponential's and the reciprocal's: below kScreenErr0 whatever b3.
+struct FxParams {
+    long long K[2];   // b0 + b1 If, plus half a unit of the high word
+    int b2, b4;
+    int b3, g3;       // b3 and b3 / sqrt(2)
+    float scale;      // -log2(e) 2^-k
+};
+
+constexpr float kFxOne = 1073741824.0f;   // 2^30
+
+__device__ __forceinline__ int fx_of(float x) { return __float2int_rn(__fmul_rn(x, kFxOne)); }
+
+// Features the fixed-point screen can take (false for NaN).
+__device__ __forceinline__ bool fx_feature(float psi, float sig, float cw, float sw)
+{
+    return fabsf(psi) <= 1.0f && fabsf(sig) < 1.99f && fabsf(cw) <= 1.0f &&
+           fabsf(sw) <= 1.0f;
+}
+
+// log2 scale of z for these coefficients; 0 when they are out of range (NaN
+// and infinities too: fmax drops a NaN, but the sum keeps it).
+__device__ __forceinline__ int fx_scale(const double b[5])
+{
+    const double mx = fmax(fmax(fabs(b[2]), fabs(b[3])), fabs(b[4]));
+    const double sum = fabs(b[0]) + fabs(b[1]) + fabs(b[2]) + 1.4143 * fabs(b[3]) +
+                       2.0 * fabs(b[4]);
+    if (mx < 63.9 && sum < 255.0) return 23;
+    return mx < 127.9 && sum < 511.0 ? 22 : 0;   // false for NaN
+}
+
+__device__ __forceinline__ void fx_fill(const double b[5], int k, FxParams &f)
+{
+    const double one = (double)(1 << (k + 2)), two30 = 1073741824.0;
+    const long long half = 1ll << 31;
+    f.K[0] = __double2ll_rn(__dmul_rn(__dmul_rn(b[0], one), two30)) + half;
+    f.K[1] = __double2ll_rn(__dmul_rn(__dmul_rn(__dadd_rn(b[0], b[1]), one), two30)) + half;
+    f.b2 = __double2int_rn(__dmul_rn(b[2], one));
+    f.b4 = __double2int_rn(__dmul_rn(b[4], one));
+    f.b3 = __double2int_rn(__dmul_rn(b[3], one));
+    f.g3 = __double2int_rn(__dmul_rn(__dmul_rn(b[3], spec::kHalfSqrt2), one));
+    f.scale = -1.44269504f / (float)(1 << k);
+}
+
+// Direction-independent part of z, without and with the slope term.
+__device__ __forceinline__ long long fx_base(const FxParams &f, bool forest, int psi)
+{
+    return f.K[forest ? 1 : 0] + (long long)f.b2 * psi;
+}
+__device__ __forceinline__ long long fx_slope(const FxParams &f, long long base, int sig)
+{
+    return base + (long long)f.b4 * sig;
+}
+
+// z of direction j of a half (0: N, NE, E, SE; the other half's directions are
+// the opposite ones, with h, g negated): acc is fx_base, or fx_slope where the
+// target lies higher; h, g are b3 and b3 / sqrt(2), c, s the wind's cosine and
+// sine.
+__device__ __forceinline__ long long fx_z(long long acc, int h, int g, int c, int s, int j)
+{
+    switch (j) {
+    case 0: return acc + (long long)h * c;
+    case 1: return acc + (long long)g * c + (long long)g * s;
+    case 2: return acc + (long long)h * s;
+    default: return acc + (long long)g * s + (long long)(-g) * c;
+    }
+}
+
+__device__ __forceinline__ float fx_p(const FxParams &f, long long z)
+{
+    float e, r;
+    asm("ex2.approx.ftz.f32 %0, %1;"
+        : "=f"(e)
+        : "f"(__fmul_rn(__int2float_rn((int)(z >> 32)), f.scale)));
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(__fadd_rn(1.0f, e)));
+    return r;
+}
+
 // Decision of the trial with draw u.  Returns 1 success, 0 failure, -1 when
 // the screen cannot decide and the exact threshold is needed.
 __device__ __forceinline__ int screen_decide(float p32, uint32_t u,

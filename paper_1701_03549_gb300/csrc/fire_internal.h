@@ -24,12 +24,15 @@ struct MapDev {
     int H, W, TH, TW, ntiles;
     const float4 *feat;         // (psi, sig, cos wind, sin wind) per cell
     const float2 *wdiag;        // cos(wind - 45 deg), cos(wind - 135 deg) per cell
-    const float2 *ps;           // (psi, sig) per cell
-    // A wind raster of one value everywhere (bit for bit) has the same four
-    // wind terms in every cell: the simulation then reads them from here and
-    // only (psi, sig) per cell (10 bytes with the flags instead of 26).
-    int uniform_wind;
-    float cw, sw, om1, om3;
+    // Fixed-point covariates of the simulation's screen (fx 0: some cell is out
+    // of their range and the float-pair screen runs).  A wind raster of one
+    // value everywhere (bit for bit) has the same cosine and sine in every
+    // cell: the simulation then reads them from here and only (psi, sig) per
+    // cell, 10 bytes with the flags; else (psi, sig, cos, sin), 18 bytes.
+    int fx, uniform_wind;
+    int cw, sw;                 // scale 2^30, uniform wind
+    const int2 *fx2;            // (psi, sig) per cell, uniform wind
+    const int4 *fx4;            // (psi, sig, cos, sin) per cell
     const uint16_t *cfl;        // bit d<8 uphill from source d, 8 forest, 9 burnable
     const uint32_t *blk;        // non-burnable bitmap, ntiles * 32 words
     const uint2 *init;          // every word of blk twice: a simulation's initial
@@ -82,6 +85,8 @@ struct SimShared {
     uint4 rk[5];          // Philox round keys: (k0, k1) of round 2j, then 2j + 1
     double beta[5];
     ScreenParams sp;
+    FxParams fx;
+    int use_fx;           // the map and the parameters fit the fixed-point screen
     uint32_t key0, key1;
     int sim;
     int skip;
@@ -131,8 +136,10 @@ __host__ __device__ inline SimLayout sim_layout(int ntiles, int qcap,
 cudaError_t launch_features(int H, int W, const uint8_t *veg, const float *elev,
                             const float *slope, const float *aspect,
                             const float *wind, float4 *feat, float2 *wdiag,
-                            float2 *ps, uint16_t *cfl, uint32_t *wind_varies,
-                            cudaStream_t st);
+                            uint16_t *cfl, uint32_t *flags, cudaStream_t st);
+// Fixed-point covariates of every cell into fx2 or fx4 (the other one NULL).
+cudaError_t launch_fx(long long n, const float4 *feat, int2 *fx2, int4 *fx4,
+                      cudaStream_t st);
 cudaError_t launch_blocked(const MapDev &m, const uint8_t *veg, uint32_t *blk,
                            uint2 *init, cudaStream_t st);
 cudaError_t launch_target(const MapDev &m, const uint8_t *burnt, uint32_t *tgt,
@@ -239,7 +246,7 @@ struct fire_map {
     float cell_m = 0.f;
     float4 *feat = nullptr;
     float2 *wdiag = nullptr;
-    float2 *ps = nullptr;
+    void *fx = nullptr;
     uint16_t *cfl = nullptr;
     uint32_t *blk = nullptr;
     uint2 *init = nullptr;

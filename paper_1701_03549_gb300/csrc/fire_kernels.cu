@@ -24,9 +24,10 @@
 //    burning source in each direction, built with shifts across tile edges;
 //    the candidates are queued and spread evenly over the warp's lanes; each
 //    candidate draws one Philox block per half of its directions (counter =
-//    (cell, step, d/4, 0), key = seed) and decides each trial through the
-//    single-precision screen, falling back to the exact double-precision
-//    threshold only near the decision boundary.
+//    (cell, step, d/4, 0), key = seed) and decides the half's trials together
+//    through a fixed-point single-precision screen (float pairs where map or
+//    coefficients are out of its range), falling back to the exact
+//    double-precision threshold only near the decision boundary.
 //  * Fused fitness: at extinction a final sweep of the planes popcounts the
 //    burnt cells and those also in the target bit plane (|A*| and |A n A*|
 //    of Eq. 2) and records whether the fire reached the grid's border.
@@ -59,9 +60,8 @@ __global__ void k_features(int H, int W, const uint8_t *__restrict__ veg,
                            const float *__restrict__ wind,
                            float4 *__restrict__ feat,
                            float2 *__restrict__ wdiag,
-                           float2 *__restrict__ ps,
                            uint16_t *__restrict__ cfl,
-                           uint32_t *__restrict__ wind_varies)
+                           uint32_t *__restrict__ flags)
 {
     const long long n = (long long)H * W;
     const uint32_t wind0 = __float_as_uint(wind[0]);
@@ -89,11 +89,24 @@ __global__ void k_features(int H, int W, const uint8_t *__restrict__ veg,
         if (v == 1) f |= kFlagForest;
         if (v != 0) f |= kFlagBurnable;
         feat[i] = make_float4(psi, sig, cw, sw);
-        ps[i] = make_float2(psi, sig);
-        if (__float_as_uint(wind[i]) != wind0) *wind_varies = 1u;
+        if (__float_as_uint(wind[i]) != wind0) flags[0] = 1u;
+        if (!fx_feature(psi, sig, cw, sw)) flags[1] = 1u;
         wdiag[i] = make_float2(__double2float_rn(spec::omega(cw, sw, 1)),
                                __double2float_rn(spec::omega(cw, sw, 3)));
         cfl[i] = f;
+    }
+}
+
+// Fixed-point covariates (FxParams): (psi, sig), or with the wind's cosine and
+// sine where it varies.
+__global__ void k_fx(long long n, const float4 *__restrict__ feat,
+                     int2 *__restrict__ fx2, int4 *__restrict__ fx4)
+{
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
+         i += (long long)gridDim.x * blockDim.x) {
+        const float4 f = feat[i];
+        if (fx2) fx2[i] = make_int2(fx_of(f.x), fx_of(f.y));
+        if (fx4) fx4[i] = make_int4(fx_of(f.x), fx_of(f.y), fx_of(f.z), fx_of(f.w));
     }
 }
 
@@ -303,29 +316,21 @@ static __device__ __noinline__ int exact_cell_decide(const double *beta,
     return (uint64_t)u < (uint64_t)floor(__dmul_rn(P, 4294967296.0)) ? 1 : 0;
 }
 
-// All trials of one candidate cell (dm: directions with a burning source).
-__device__ __forceinline__ bool trial_cell(const SimCtx &s, uint32_t cell,
-                                           uint32_t dm, uint32_t t)
+// All trials of one candidate cell through the float-pair screen (maps or
+// parameters out of the fixed-point range).
+static __device__ __noinline__ bool trial_cell_ff(const MapDev &m, const SimShared &sh,
+                                                  bool cell_uniform, uint32_t cell,
+                                                  uint32_t dm, uint32_t t)
 {
-    const MapDev &m = *s.map;
-    const SimShared &sh = *s.sh;
-    float4 f;   // (psi, sig, cos wind, sin wind)
-    float2 wd;  // diagonal wind terms
-    if (m.uniform_wind) {
-        const float2 p = __ldg(&m.ps[cell]);
-        f = make_float4(p.x, p.y, m.cw, m.sw);
-        wd = make_float2(m.om1, m.om3);
-    } else {
-        f = __ldg(&m.feat[cell]);
-        wd = __ldg(&m.wdiag[cell]);
-    }
+    const float4 f = __ldg(&m.feat[cell]);     // (psi, sig, cos wind, sin wind)
+    const float2 wd = __ldg(&m.wdiag[cell]);   // diagonal wind terms
     const uint32_t fl = __ldg(&m.cfl[cell]);
     const bool forest = (fl & kFlagForest) != 0;
     const uint32_t up = fl & 0xffu;
     const ScreenCell sc = screen_cell(sh.sp, forest, f.x, f.y, f.z, wd.x, f.w,
                                       wd.y);
     const ff b3 = sh.sp.b3;
-    if (s.a->cell_uniform) {
+    if (cell_uniform) {
         float q = 1.0f;
         uint32_t mm = dm;
         while (mm) {
@@ -339,21 +344,112 @@ __device__ __forceinline__ bool trial_cell(const SimCtx &s, uint32_t cell,
         if (dec < 0) dec = exact_cell_decide(sh.beta, forest, f, up, dm, u);
         return dec != 0;
     }
-    // The cell ignites iff any trial succeeds, whatever the order they are
-    // tested in; the half with more burning sources goes first, so that the
-    // second Philox block is needed less often.
-    const uint32_t lo = dm & 0x0fu, hi = dm >> 4;
-    const uint32_t first = __popc(hi) > __popc(lo) ? 1u : 0u;
     bool ign = false;
-    for (uint32_t k = 0; k < 2 && !ign; ++k) {
-        const uint32_t half = first ^ k;
-        const uint32_t m4 = half ? hi : lo;
+    for (uint32_t half = 0; half < 2 && !ign; ++half) {
+        const uint32_t m4 = half ? dm >> 4 : dm & 0x0fu;
         if (!m4) continue;
         const uint4 u = philox4x32_10_rk(cell, t, half, 0u, sh.rk);
         ign = test_dirs(m4, (int)(half * 4), u, sc, b3, sh.sp.margin, up,
                         sh.beta, forest, f);
     }
     return ign;
+}
+
+// Exact decisions of a cell of the fixed-point screen (the double-precision
+// definition reads the float covariates): any trial of the directions in m4
+// (bit j: direction base + j), drawn from one Philox block.
+static __device__ __noinline__ bool exact_half_at(const MapDev &m, const double *beta,
+                                                  uint32_t cell, uint32_t m4, int base,
+                                                  uint4 u4)
+{
+    const uint32_t fl = __ldg(&m.cfl[cell]);
+    const float4 f = __ldg(&m.feat[cell]);
+    const uint32_t u[4] = {u4.x, u4.y, u4.z, u4.w};
+    for (int j = 0; j < 4; ++j) {
+        const int d = base + j;
+        if (((m4 >> j) & 1u) && exact_decide(beta, (fl & kFlagForest) != 0, f,
+                                             (fl >> d) & 1u, d, u[j]))
+            return true;
+    }
+    return false;
+}
+static __device__ __noinline__ int exact_cell_at(const MapDev &m, const double *beta,
+                                                 uint32_t cell, uint32_t dm, uint32_t u)
+{
+    const uint32_t fl = __ldg(&m.cfl[cell]);
+    return exact_cell_decide(beta, (fl & kFlagForest) != 0, __ldg(&m.feat[cell]),
+                             fl & 0xffu, dm, u);
+}
+
+// All trials of one candidate cell (dm: directions with a burning source).
+__device__ __forceinline__ bool trial_cell(const SimCtx &s, uint32_t cell,
+                                           uint32_t dm, uint32_t t)
+{
+    const MapDev &m = *s.map;
+    const SimShared &sh = *s.sh;
+    if (!sh.use_fx) return trial_cell_ff(m, sh, s.a->cell_uniform != 0, cell, dm, t);
+    int psi, sig, c, sn;   // sn: sine of the wind
+    if (m.uniform_wind) {
+        const int2 p = __ldg(&m.fx2[cell]);
+        psi = p.x;
+        sig = p.y;
+        c = m.cw;
+        sn = m.sw;
+    } else {
+        const int4 p = __ldg(&m.fx4[cell]);
+        psi = p.x;
+        sig = p.y;
+        c = p.z;
+        sn = p.w;
+    }
+    const uint32_t fl = __ldg(&m.cfl[cell]);
+    const FxParams &fx = sh.fx;
+    const long long acc = fx_base(fx, (fl & kFlagForest) != 0, psi);
+    const long long accg = fx_slope(fx, acc, sig);
+    if (s.a->cell_uniform) {
+        float q = 1.0f;
+#pragma unroll
+        for (int d = 0; d < 8; ++d) {
+            const int h = d < 4 ? fx.b3 : -fx.b3, g = d < 4 ? fx.g3 : -fx.g3;
+            const float p = fx_p(fx, fx_z((fl >> d) & 1u ? accg : acc, h, g, c, sn, d & 3));
+            if ((dm >> d) & 1u) q = __fmul_rn(q, __fsub_rn(1.0f, p));
+        }
+        const uint32_t u = philox4x32_10_rk(cell, t, 2u, 0u, sh.rk).x;
+        int dec = screen_decide(__fsub_rn(1.0f, q), u, sh.sp.cell_margin);
+        if (dec < 0) dec = exact_cell_at(m, sh.beta, cell, dm, u);
+        return dec != 0;
+    }
+    // The cell ignites iff any trial succeeds, whatever the order they are
+    // tested in; the half with more burning sources goes first, so that the
+    // second Philox block is needed less often.  The four directions of a half
+    // are evaluated together, whether or not a source burns there: four
+    // independent chains take little longer than one (a loop over the set
+    // bits costs the warp one chain per trial of its busiest lane).
+    const uint32_t lo = dm & 0x0fu, hi = dm >> 4;
+    const uint32_t first = __popc(hi) > __popc(lo) ? 1u : 0u;
+    for (uint32_t k = 0; k < 2; ++k) {
+        const uint32_t half = first ^ k;
+        const uint32_t m4 = half ? hi : lo;
+        if (!m4) continue;
+        const uint4 u4 = philox4x32_10_rk(cell, t, half, 0u, sh.rk);
+        const uint32_t u[4] = {u4.x, u4.y, u4.z, u4.w};
+        const int h = half ? -fx.b3 : fx.b3, g = half ? -fx.g3 : fx.g3;
+        const uint32_t up = fl >> (half * 4);
+        // the largest p - (u + 1) 2^-32 decides unless it is near zero
+        float best = -2.0f;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const float p = fx_p(fx, fx_z((up >> j) & 1u ? accg : acc, h, g, c, sn, j));
+            const float v = __fmaf_rn(__uint2float_rn(u[j]), 0x1p-32f, 0x1p-32f);
+            const float diff = __fsub_rn(p, v);
+            if ((m4 >> j) & 1u) best = fmaxf(best, diff);
+        }
+        if (best > sh.sp.margin) return true;
+        if (best >= -sh.sp.margin &&
+            exact_half_at(m, sh.beta, cell, m4, (int)(half * 4), u4))
+            return true;
+    }
+    return false;
 }
 
 // Cell (row r, column i of tile k = (ti, tj)) ignites at step t: write it with
@@ -663,6 +759,9 @@ __global__ void __launch_bounds__(kSimMaxThreads, 2) k_simulate(SimLaunch a)
             const fire_params P = a.params[sim];
             for (int j = 0; j < 5; ++j) sh.beta[j] = P.b[j];
             sh.sp = screen_params(P.b);
+            const int k = sh.map.fx ? fx_scale(P.b) : 0;
+            sh.use_fx = k;
+            if (k) fx_fill(P.b, k, sh.fx);
             const uint64_t seed = a.seeds[sim];
             sh.key0 = (uint32_t)seed;
             sh.key1 = (uint32_t)(seed >> 32);
@@ -1003,6 +1102,23 @@ __global__ void k_thresholds(MapDev m, const double *__restrict__ beta_dev,
     }
 }
 
+// p32 as the simulation's screen computes it: fixed point with z's scale k, or
+// float pairs (k = 0).
+__device__ float screen_any(const double b[5], const ScreenParams &sp, int k, bool forest,
+                            float4 f, float om1, float om3, bool up, int d)
+{
+    if (!k) {
+        const ScreenCell sc = screen_cell(sp, forest, f.x, f.y, f.z, om1, f.w, om3);
+        return screen_p(screen_z(sc, sp.b3, up, d));
+    }
+    FxParams fx;
+    fx_fill(b, k, fx);
+    const long long acc = fx_base(fx, forest, fx_of(f.x));
+    const int h = d < 4 ? fx.b3 : -fx.b3, g = d < 4 ? fx.g3 : -fx.g3;
+    return fx_p(fx, fx_z(up ? fx_slope(fx, acc, fx_of(f.y)) : acc, h, g, fx_of(f.z),
+                         fx_of(f.w), d & 3));
+}
+
 __global__ void k_probabilities(MapDev m, const double *__restrict__ beta_dev,
                                 float *__restrict__ p32,
                                 double *__restrict__ p64)
@@ -1011,6 +1127,7 @@ __global__ void k_probabilities(MapDev m, const double *__restrict__ beta_dev,
     double b[5];
     for (int j = 0; j < 5; ++j) b[j] = beta_dev[j];
     const ScreenParams sp = screen_params(b);
+    const int k = m.fx ? fx_scale(b) : 0;
     for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
          idx < 8 * HW; idx += (long long)gridDim.x * blockDim.x) {
         const int d = (int)(idx / HW);
@@ -1020,9 +1137,7 @@ __global__ void k_probabilities(MapDev m, const double *__restrict__ beta_dev,
         const bool forest = fl & kFlagForest, up = (fl >> d) & 1u;
         if (p32) {
             const float2 wd = m.wdiag[i];
-            const ScreenCell sc =
-                screen_cell(sp, forest, f.x, f.y, f.z, wd.x, f.w, wd.y);
-            p32[idx] = screen_p(screen_z(sc, sp.b3, up, d));
+            p32[idx] = screen_any(b, sp, k, forest, f, wd.x, wd.y, up, d);
         }
         if (p64)
             p64[idx] = spec::logistic(
@@ -1095,20 +1210,25 @@ __global__ void k_screen_selftest(uint64_t n, uint64_t seed,
         const ScreenParams sp = screen_params(b);
         const float om1 = __double2float_rn(spec::omega(cw, sw, 1));
         const float om3 = __double2float_rn(spec::omega(cw, sw, 3));
-        const ScreenCell sc = screen_cell(sp, forest, psi, sig, cw, om1, sw, om3);
-        const float p32 = screen_p(screen_z(sc, sp.b3, up, d));
-        int dec = screen_decide(p32, u, sp.margin);
         const bool exact = (uint64_t)u < T;
         local[0]++;
-        if (dec < 0) {
-            local[1]++;
-            dec = exact;
+        // both screens where the fixed-point one applies: the simulation runs
+        // one or the other
+        const int k = fx_feature(psi, sig, cw, sw) ? fx_scale(b) : 0;
+        for (int which = k ? 0 : 1; which < 2; ++which) {
+            const float p32 = screen_any(b, sp, which ? 0 : k, forest,
+                                         make_float4(psi, sig, cw, sw), om1, om3, up, d);
+            int dec = screen_decide(p32, u, sp.margin);
+            if (dec < 0) {
+                if (which == (k ? 0 : 1)) local[1]++;
+                dec = exact;
+            }
+            if ((dec != 0) != exact) local[2]++;
+            // |p32 - p64| against the screen's stated bound
+            const double dp = fabs((double)p32 - spec::logistic(z));
+            local_max = fmax(local_max,
+                             dp / ((double)kScreenErrB3 * fabs(b[3]) + kScreenErr0));
         }
-        if ((dec != 0) != exact) local[2]++;
-        // |p32 - p64| against the screen's stated bound
-        const double dp = fabs((double)p32 - spec::logistic(z));
-        local_max = fmax(local_max,
-                         dp / ((double)kScreenErrB3 * fabs(b[3]) + kScreenErr0));
     }
     for (int j = 0; j < 3; ++j) {
         unsigned long long v = local[j];
@@ -1192,15 +1312,20 @@ static int grid_for(long long n, int block)
 cudaError_t launch_features(int H, int W, const uint8_t *veg, const float *elev,
                             const float *slope, const float *aspect,
                             const float *wind, float4 *feat, float2 *wdiag,
-                            float2 *ps, uint16_t *cfl, uint32_t *wind_varies,
-                            cudaStream_t st)
+                            uint16_t *cfl, uint32_t *flags, cudaStream_t st)
 {
     const long long n = (long long)H * W;
-    cudaError_t e = cudaMemsetAsync(wind_varies, 0, sizeof(uint32_t), st);
+    cudaError_t e = cudaMemsetAsync(flags, 0, 2 * sizeof(uint32_t), st);
     if (e != cudaSuccess) return e;
     k_features<<<grid_for(n, 256), 256, 0, st>>>(H, W, veg, elev, slope, aspect,
-                                                 wind, feat, wdiag, ps, cfl,
-                                                 wind_varies);
+                                                 wind, feat, wdiag, cfl, flags);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_fx(long long n, const float4 *feat, int2 *fx2, int4 *fx4,
+                      cudaStream_t st)
+{
+    k_fx<<<grid_for(n, 256), 256, 0, st>>>(n, feat, fx2, fx4);
     return cudaGetLastError();
 }
 
