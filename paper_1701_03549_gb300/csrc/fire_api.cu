@@ -85,12 +85,33 @@ bool valid_map(const fire_map *m) { return m && m->ctx && m->feat; }
 
 // Launch shape of the simulation kernel for maps of up to `ntiles` tiles:
 // an explicit fire_set_launch override, else the autotuned shape recorded for
-// this tile count, else a heuristic.
-int plan_launch(fire_ctx *ctx, int ntiles, long long n, LaunchPlan *p, bool burn)
+// this tile count, else a rule on the map and the batch.
+//
+// The rule (ms on one GB300; q fires per SM of 152).  A fire runs faster in a
+// block of many warps, a full SM does more with many blocks of few: with q
+// below 8 the launch is as long as its longest fires and wide blocks win
+// (512 x 512, q = 1: 16 warps 3.2, 8 warps 4.5, 4 warps 6.9; q = 4: 7.0, 6.7,
+// 9.9), from there on four blocks of 8 warps with their state in global memory
+// (1024 x 1024 generation, q = 27: 13.3 against 17.1 at 16 warps; nine uneven
+// fires, q = 118: 276 against 318), and with many fires of up to 1024 tiles
+// eight blocks of 4 warps (512 x 512 generation, q = 27: 22.0 against 22.5 at 8
+// warps and 24.4 at 16; ignition search, q = 108: 46 against 54 and 75).  Up to
+// 64 tiles the shared-memory shapes stay within a few per cent of these.  A
+// shared-memory state of which only one block fits an SM (about 400 to 700
+// tiles) is worth it for at most one fire per SM (801 x 801, q = 7: 17.1 shared,
+// 13.4 in global memory with two blocks).  The burn-time variant has no shared
+// state (256 x 256, q = 4: 4.3 at 8 warps, 5.5 at 4; 512 x 512, q = 13: 29.0
+// and 28.3).
+//
+// fixed_scratch: the caller cannot provide a state buffer per block, so a state
+// that fits in shared memory goes there.
+int plan_launch(fire_ctx *ctx, int ntiles, long long n, LaunchPlan *p, bool burn,
+                bool fixed_scratch)
 {
     int warps = 0, bps = 0, queue = 0, state = FIRE_STATE_AUTO;
     const bool override = ctx->warps_per_block || ctx->blocks_per_sm ||
                           ctx->queue_entries || ctx->state_mode;
+    bool tuned = false;
     if (override) {
         warps = ctx->warps_per_block;
         bps = ctx->blocks_per_sm;
@@ -103,21 +124,33 @@ int plan_launch(fire_ctx *ctx, int ntiles, long long n, LaunchPlan *p, bool burn
                 bps = t.bps;
                 queue = t.queue;
                 state = t.state;
+                tuned = true;
             }
         }
+        // the burn-time variant cannot use a shape tuned for shared state
+        if (burn && state != FIRE_STATE_GLOBAL) tuned = false;
+    }
+    if (!override && !tuned && (burn || (ntiles > 64 && !fixed_scratch))) {
+        const long long sms = ctx->num_sms;
+        const size_t shared = sim_layout(ntiles, 4096, true).total;
+        if (n >= (burn ? 12 : 24) * sms && ntiles <= 1024) {
+            warps = 4, bps = 8, queue = burn ? 3072 : 2048, state = FIRE_STATE_GLOBAL;
+        } else if (n >= (burn ? 2 : 8) * sms) {
+            warps = 8, bps = 4, queue = 3072, state = FIRE_STATE_GLOBAL;
+        } else if (burn || ntiles > 1024 ||
+                   (n > sms && 2 * (shared + 1024) > ctx->smem_per_sm &&
+                    shared <= ctx->max_smem_optin)) {
+            warps = 16, bps = 2, queue = 8192, state = FIRE_STATE_GLOBAL;
+        }
+        // long worklists take the room of the larger queues
+        if (state == FIRE_STATE_GLOBAL &&
+            sim_layout(ntiles, queue, false).total > ctx->max_smem_optin)
+            queue = 0;
     }
     int nwarps = warps > 0 ? warps : (ntiles <= 16 ? 4 : (ntiles <= 64 ? 8 : 16));
     nwarps = std::min(nwarps, kSimMaxThreads / 32);
     int qcap = queue > 0 ? queue : 4096;
     SimLayout L = sim_layout(ntiles, qcap, true);
-    // the burn-time variant keeps its state in global memory; a shape tuned
-    // for shared-memory state gives way to the global-state shape that is
-    // fastest on the plain kernel's benchmarks (4 warps x 8 blocks per SM)
-    if (burn && !override && state != FIRE_STATE_GLOBAL) {
-        nwarps = 4;
-        bps = 8;
-        qcap = queue = 3072;
-    }
     if (burn) state = FIRE_STATE_GLOBAL;
     bool smem_state = state == FIRE_STATE_SHARED ||
                       (state == FIRE_STATE_AUTO && L.total <= ctx->max_smem_optin);
@@ -179,6 +212,7 @@ int fire_create(fire_ctx **out, int device, void *cuda_stream)
     if (e != cudaSuccess) { delete ctx; return FIRE_ECUDA; }
     ctx->num_sms = prop.multiProcessorCount;
     ctx->max_smem_optin = prop.sharedMemPerBlockOptin;
+    ctx->smem_per_sm = prop.sharedMemPerMultiprocessor;
     if (cuda_stream) {
         ctx->stream = (cudaStream_t)cuda_stream;
     } else {

@@ -210,7 +210,7 @@ struct GraphEntry {
 struct fire_ctx {
     int device = 0;
     int num_sms = 0;
-    size_t max_smem_optin = 0;
+    size_t max_smem_optin = 0, smem_per_sm = 0;
     cudaStream_t stream = nullptr;
     bool own_stream = false;
     int warps_per_block = 0;   // 0: heuristic
@@ -267,9 +267,10 @@ size_t round16(size_t x);
 bool valid_map(const fire_map *m);
 int noalloc_take_error(int device, bool *set);
 // Launch shape of the simulation kernel (burn: the burn-time variant, whose
-// state is always in global memory).
+// state is always in global memory; fixed_scratch: no state buffer can be
+// grown, so a state that fits in shared memory goes there).
 int plan_launch(fire_ctx *ctx, int ntiles, long long n, LaunchPlan *p,
-                bool burn = false);
+                bool burn = false, bool fixed_scratch = false);
 cudaError_t launch_conv_tma(int mode, const uint16_t *in, const uint16_t *w,
                             const float *bias, const uint16_t *hprev, uint16_t *out,
                             int n, int S, int lgS, int d, uint32_t *err,

@@ -146,10 +146,11 @@ extern "C" int fire_simulate_batch_noalloc(fire_ctx *ctx, const fire_map *m,
     int rc = scratch_address(ctx, ctx->device, &scratch);
     if (rc) return rc;
 
-    // launch shape, as fire_simulate_batch chooses it
+    // launch shape: as fire_simulate_batch chooses it, but for its rules that
+    // trade shared-memory state for more blocks with buffers of their own
     const int ntiles = m->dev.ntiles;
     LaunchPlan plan;
-    rc = plan_launch(ctx, ntiles, n, &plan);
+    rc = plan_launch(ctx, ntiles, n, &plan, false, true);
     if (rc) return rc;
     const bool smem_state = plan.smem_state;
     long long grid = plan.grid;
