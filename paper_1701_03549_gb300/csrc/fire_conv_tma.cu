@@ -1,7 +1,7 @@
 // TMA-fed implicit-GEMM convolutions of the surrogate network on tcgen05
 // tensor cores: the 128 -> 128 layers forward and input gradient
-// (k_conv_pair), their weight gradient (k_wgrad_tma) and the first layer
-// forward (k_conv1_tma).
+// (k_conv_pair), the weight and bias gradients of all layers (k_wgrad_strip)
+// and the first layer forward (k_conv1_tma).
 //
 // In each, one thread issues tensor-map copies of shifted NHWC activation
 // boxes (channels, x, y, sample; out-of-range elements read as zero, which is
@@ -24,18 +24,7 @@
 namespace fire {
 namespace convtma {
 
-constexpr int kTileBytes = 128 * 128;           // 128 rows x 64 BF16
-constexpr int kStageBytes = 2 * kTileBytes;     // A + B
 constexpr int kSlabs = 18;                      // 9 taps x 2 channel halves
-// The weight-gradient kernel's own stage count and residency.
-#ifndef FIRE_WGRAD_STAGES
-#define FIRE_WGRAD_STAGES 2
-#endif
-constexpr int kWStages = FIRE_WGRAD_STAGES;
-constexpr int kWSmem = kWStages * kStageBytes + 1024;
-constexpr int kWCtasPerSm =
-    (227 * 1024) / (kWSmem + 2048) > 4 ? 4 : (227 * 1024) / (kWSmem + 2048);
-
 struct Epi {
     int mode;                 // 0 forward (bias + ReLU), 1 input gradient (mask)
     const float *bias;        // forward
@@ -510,129 +499,237 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
     if (warp == kEpiWarps) tmem_dealloc_pair(tmem, 256);
 }
 
-// Weight gradient of a 128 -> 128 layer: D[o][(t, i)] = sum_p dz[p, o]
-// in[p + off(t), i].  CTA (tap t = blockIdx.y, pixel range blockIdx.z) runs
-// 64-pixel slabs; both operands are MN-major (8 consecutive channels per 16
-// bytes, pixels along K).  Each slab is two 64-channel TMA boxes per operand,
-// which land as the MN-major SWIZZLE_128B layout: channel halves 8 KB apart
-// (LBO), 8-pixel groups 1 KB apart (SBO).  Partial sums are added to dW with
-// FP32 atomics.
-__device__ __forceinline__ uint64_t desc_sw128_mn(uint32_t saddr)
+// Weight and bias gradients of a layer of Cin input channels (128 or 16):
+// dW[o][(t, i)] += sum_p dz[p, o] in[p + off(t), i], db[o] += sum_p dz[p, o].
+// Both operands are MN-major (channels within 128 or 32 bytes of a pixel,
+// pixels along K).  A slab is L pixels: dz, and strips of `in` with d pixels
+// on either side of each row, so that the three taps of a row of taps are one
+// operand: N = 3 taps x 64 (16) channels, the taps d pixels apart (the
+// leading-dimension stride; swizzles go by address, so a tap may start at any
+// pixel).  Where a strip of separate rows would be wider than three boxes
+// (d >= S) it is three boxes, one per tap.  A CTA takes a range of slabs and,
+// with 128 channels, one row of taps and both channel halves (2 x N = 192),
+// with 16 all three rows (3 x N = 48); a column of ones beside them gives the
+// bias gradient in the same pass, shared out over the rows' CTAs.
+//
+// What bounds it (128 channels, 8 x 256 x 256, 154.6 GFLOP): shared memory,
+// which a 128 x 192 x 16 MMA reads at 107 bytes a clock (128 x 128 x 16: 128)
+// while the copies write 45.  98.5 us with the bias (d = 64: 103); one tap per
+// CTA with a box per operand loaded 32 KB per 64 pixels and tap: 119 us, and
+// another 27 us for a bias pass over dz.  16 channels: 31 us (bound by reading
+// dz, 134 MB) against 204 on register-staged tiles.
+struct WgradShape {
+    int L, lgw;        // pixels of a slab, log2 pixels of its rows
+    int pitch;         // pixels from one row of a strip to the next
+    int nbox, box;     // boxes of a strip and the bytes of one
+    int tap;           // bytes from one tap to the next
+    int strip, stages;
+};
+
+constexpr int kMaxWgStages = 6;
+constexpr int kWgThreads = 192;
+constexpr int kOnesBytes = 2048;
+constexpr int kWgRoom = 227 * 1024 - 2048 - kOnesBytes;   // beside alignment, barriers
+
+struct WgradShared {
+    unsigned long long full[kMaxWgStages], empty[kMaxWgStages], done;
+    uint32_t tmem_slot;
+    int fail, issued, used;
+};
+
+__device__ __forceinline__ uint64_t desc_mn(uint32_t saddr, uint32_t lbo, uint32_t sbo,
+                                            uint32_t swizzle)
 {
     uint64_t d = (uint64_t)((saddr & 0x3ffffu) >> 4);
-    d |= (uint64_t)(8192 >> 4) << 16;       // LBO: next 64 MN elements
-    d |= (uint64_t)(1024 >> 4) << 32;       // SBO: next 8 K rows
+    d |= (uint64_t)(lbo >> 4) << 16;        // next 64 (16) MN elements
+    d |= (uint64_t)(sbo >> 4) << 32;        // next 8 K rows
     d |= (uint64_t)1 << 46;
-    d |= (uint64_t)2 << 61;                 // SWIZZLE_128B
+    d |= (uint64_t)swizzle << 61;           // 2: 128 bytes, 6: 32 bytes
     return d;
 }
 
-__global__ void __launch_bounds__(128, kWCtasPerSm)
-    k_wgrad_tma(const __grid_constant__ CUtensorMap dzm,
-                const __grid_constant__ CUtensorMap inm, float *dw, int S, int lgS,
-                int d, int slabs_total, int slabs_per, uint32_t *err)
+template <int Cin, int kSteps>
+__global__ void __launch_bounds__(kWgThreads, 1)
+    k_wgrad_strip(const __grid_constant__ CUtensorMap dzm,
+                  const __grid_constant__ CUtensorMap inm, float *dw, float *db, int S,
+                  int lgS, int d, WgradShape sp, int slabs_total, int slabs_per,
+                  uint32_t *err)
 {
+    constexpr int kB = Cin == 128 ? 2 : 3;          // strips of a slab
+    constexpr int kCh = Cin == 128 ? 64 : 16;       // channels of a strip
+    constexpr int kN = 3 * kCh;
+    constexpr uint32_t kRow = kCh * 2;              // bytes of a pixel
+    constexpr uint32_t kSwizzle = Cin == 128 ? 2 : 6;
+    constexpr int kBiasCol = kB * kN;
+    constexpr int kCols = Cin == 128 ? 512 : 256;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
-    __shared__ __align__(8) unsigned long long full[kWStages], empty[kWStages], done;
-    __shared__ uint32_t tmem_slot;
-    __shared__ int s_fail, s_issued, s_consumed;
+    const uint32_t raw = tc::smem_addr(smem_raw);
+    const uint32_t base = (raw + 1023u) & ~1023u;
+    unsigned char *const sm = smem_raw + (base - raw);
+    WgradShared &sh = *reinterpret_cast<WgradShared *>(sm + kWgRoom + kOnesBytes);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const uint32_t base = (tc::smem_addr(smem_raw) + 1023u) & ~1023u;
-    const int tap = blockIdx.y;
-    const int dy = (tap / 3 - 1) * d, dx = (tap % 3 - 1) * d;
-    const int s0 = blockIdx.z * slabs_per;
+    constexpr uint32_t kDz = kSteps * 16 * 256;     // bytes of a dz slab
+    const uint32_t stage = kDz + kB * (uint32_t)sp.strip;
+    const int dyi = Cin == 128 ? (int)blockIdx.y : 0;
+    const int s0 = blockIdx.x * slabs_per;
     const int ns = min(slabs_total - s0, slabs_per);
+    // slabs whose bias this CTA sums: all, or those of its residue mod 3
+    const int nbias = Cin == 128 ? (s0 + ns + 2 - dyi) / 3 - (s0 + 2 - dyi) / 3 : ns;
 
-    if (warp == 0) {
-        tc::tmem_alloc(&tmem_slot, 128);
+    if (warp == 4) {
+        tc::tmem_alloc(&sh.tmem_slot, kCols);
         tc::tmem_relinquish();
     }
+    for (int i = tid; i < kOnesBytes / 4; i += kWgThreads)
+        reinterpret_cast<uint32_t *>(sm + kWgRoom)[i] = 0x3f803f80u;
+    tc::fence_proxy_async();
     if (tid == 0) {
-        for (int i = 0; i < kWStages; ++i) {
-            tc::mbar_init(&full[i], 1);
-            tc::mbar_init(&empty[i], 1);
+        for (int i = 0; i < kMaxWgStages; ++i) {
+            tc::mbar_init(&sh.full[i], 1);
+            tc::mbar_init(&sh.empty[i], 1);
         }
-        tc::mbar_init(&done, 1);
-        s_fail = 0;
-        s_issued = 0;
-        s_consumed = 0;
+        tc::mbar_init(&sh.done, 1);
+        sh.fail = sh.issued = sh.used = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
-    const uint32_t tmem = tmem_slot;
+    const uint32_t tmem = sh.tmem_slot;
 
-    if (ns > 0 && warp == 0 && lane == 0) {
-        int s = 0;
+    if (warp == 4) {
+        const bool leader = elect_one();
+        int st = 0, s = 0;
+        uint32_t ph = 1;
+        bool ok = true;
         for (; s < ns; ++s) {
-            const int st = s % kWStages;
-            if (s >= kWStages &&
-                !tc::mbar_wait_bounded(&empty[st], ((s / kWStages) - 1) & 1)) {
-                atomicOr(&s_fail, 1);
-                break;
+            if (s >= sp.stages) ok = all_ok(tc::mbar_wait_bounded(&sh.empty[st], ph));
+            ok = all_ok(ok && !*(volatile int *)&sh.fail);
+            if (!ok) break;
+            if (leader) {
+                const int p0 = (s0 + s) * (kSteps * 16);
+                const int b = p0 >> (2 * lgS);
+                const int y = (p0 >> lgS) & (S - 1), x = p0 & (S - 1);
+                const uint32_t sa = base + st * stage;
+                expect_tx(&sh.full[st], kDz + kB * sp.nbox * sp.box);
+                tma_4d(sa, &dzm, 0, x, y, b, &sh.full[st]);
+                tma_4d(sa + kDz / 2, &dzm, 64, x, y, b, &sh.full[st]);
+                for (int i = 0; i < kB; ++i) {
+                    const int c = Cin == 128 ? 64 * i : 0;
+                    const int yi = y + (Cin == 128 ? dyi - 1 : i - 1) * d;
+                    for (int t = 0; t < sp.nbox; ++t)
+                        tma_4d(sa + kDz + i * sp.strip + t * sp.box, &inm, c,
+                               x + (t - 1) * d, yi, b, &sh.full[st]);
+                }
             }
-            if (*(volatile int *)&s_fail) break;
-            const int p0 = (s0 + s) * 64;
-            const int b = p0 >> (2 * lgS);
-            const int y = (p0 >> lgS) & (S - 1), x = p0 & (S - 1);
-            const uint32_t sa = base + st * kStageBytes, sb = sa + kTileBytes;
-            expect_tx(&full[st], kStageBytes);
-            tma_4d(sa, &dzm, 0, x, y, b, &full[st]);
-            tma_4d(sa + 8192, &dzm, 64, x, y, b, &full[st]);
-            tma_4d(sb, &inm, 0, x + dx, y + dy, b, &full[st]);
-            tma_4d(sb + 8192, &inm, 64, x + dx, y + dy, b, &full[st]);
+            __syncwarp();
+            if (++st == sp.stages) st = 0, ph ^= 1;
         }
-        s_issued = s;
-    } else if (ns > 0 && warp == 1 && lane == 0) {
-        constexpr uint32_t idesc =
-            tc::idesc_bf16(128, 128) | (1u << 15) | (1u << 16);   // both MN-major
-        int s = 0;
-        for (; s < ns; ++s) {
-            const int st = s % kWStages;
-            if (!tc::mbar_wait_bounded(&full[st], (s / kWStages) & 1)) {
-                atomicOr(&s_fail, 1);
-                break;
-            }
-            tc::fence_after_sync();
-            const uint32_t sa = base + st * kStageBytes, sb = sa + kTileBytes;
+        if (leader) {
+            if (!ok) atomicOr(&sh.fail, 1);
+            sh.issued = s;
+        }
+        __syncwarp();
+    } else if (warp == 5) {
+        constexpr uint32_t idesc = tc::idesc_bf16(128, kN) | (1u << 15) | (1u << 16);
+        constexpr uint32_t idesc1 = tc::idesc_bf16(128, 16) | (1u << 15) | (1u << 16);
+        const uint64_t ad = desc_mn(base, kDz / 2, 1024, 2);
+        const uint64_t bd = desc_mn(base + kDz, sp.tap, 8 * kRow, kSwizzle);
+        const uint64_t od = desc_mn(base + kWgRoom, 1024, 1024, 2);
+        const uint32_t strip16 = (uint32_t)sp.strip >> 4;
+        uint32_t row16[kSteps];   // first pixel of each 16 within a strip
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk)
-                tc::mma_bf16(tmem, desc_sw128_mn(sa + kk * 2048),
-                             desc_sw128_mn(sb + kk * 2048), idesc, s > 0 || kk > 0);
-            tc::mma_commit(&empty[st]);
+        for (int j = 0; j < kSteps; ++j)
+            row16[j] = (uint32_t)(((16 * j) >> sp.lgw) * sp.pitch +
+                                  ((16 * j) & ((1 << sp.lgw) - 1))) * (kRow / 16);
+        const bool leader = elect_one();
+        int st = 0, s = 0, nb = 0;
+        uint32_t ph = 0;
+        bool ok = true;
+        for (; s < ns; ++s) {
+            ok = all_ok(tc::mbar_wait_bounded(&sh.full[st], ph));
+            if (!ok) break;
+            tc::fence_after_sync();
+            const uint32_t off = (uint32_t)st * (stage >> 4);
+            const bool bias = Cin != 128 || (s0 + s) % 3 == dyi;
+            if (leader) {
+#pragma unroll
+                for (int j = 0; j < kSteps; ++j) {
+#pragma unroll
+                    for (int i = 0; i < kB; ++i)
+                        tc::mma_bf16(tmem + i * kN, ad + off + j * 128,
+                                     bd + off + i * strip16 + row16[j], idesc,
+                                     s > 0 || j > 0);
+                    if (bias)
+                        tc::mma_bf16(tmem + kBiasCol, ad + off + j * 128, od, idesc1,
+                                     nb > 0 || j > 0);
+                }
+                tc::mma_commit(&sh.empty[st]);
+            }
+            __syncwarp();
+            nb += bias;
+            if (++st == sp.stages) st = 0, ph ^= 1;
         }
-        s_consumed = s;
-        if (s == ns) tc::mma_commit(&done);
+        if (leader) {
+            if (!ok) atomicOr(&sh.fail, 1);
+            sh.used = s;
+            tc::mma_commit(&sh.done);   // arrives once every issued MMA is done
+        }
+        __syncwarp();
     }
-    __syncwarp();
-    if (ns > 0 && !tc::mbar_wait_bounded(&done, 0)) atomicOr(&s_fail, 1);
+    if (!tc::mbar_wait_bounded(&sh.done, 0)) atomicOr(&sh.fail, 1);
     __syncthreads();
     tc::fence_after_sync();
 
-    if (ns > 0 && !s_fail) {
-        const int o = warp * 32 + lane;
-        // 16-byte aligned: dw, the row stride (1152 floats) and tap * 128 are
-        // multiples of four floats
-        float4 *row = reinterpret_cast<float4 *>(dw + (size_t)o * 1152 + tap * 128);
+    if (ns > 0 && !sh.fail) {
+        // kPiece columns at a time through shared memory (the stages are free),
+        // so that a warp's atomics cover whole sectors
+        constexpr int kPiece = Cin == 128 ? 64 : kN;
+        constexpr int kLd = kPiece + 4;
+        float *stg = reinterpret_cast<float *>(sm);
+        const uint32_t lanes = tmem + ((uint32_t)(warp * 32) << 16);
 #pragma unroll 1
-        for (int c0 = 0; c0 < 128; c0 += 32) {
-            float v[32];
-            tc::tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
+        for (int q = 0; q < kB * kN / kPiece; ++q) {
+            if (warp < 4) {
+                float *row = stg + (warp * 32 + lane) * kLd;
+                float v[32];
+                tc::tmem_ld32(lanes + q * kPiece, v);
 #pragma unroll
-            for (int j = 0; j < 8; ++j)
-                atomicAdd(row + c0 / 4 + j,
-                          make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]));
+                for (int j = 0; j < 8; ++j)
+                    *reinterpret_cast<float4 *>(row + 4 * j) =
+                        make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+                if (Cin == 128) tc::tmem_ld32(lanes + q * kPiece + 32, v);
+                else tc::tmem_ld16(lanes + q * kPiece + 32, v);
+#pragma unroll
+                for (int j = 0; j < (kPiece - 32) / 4; ++j)
+                    *reinterpret_cast<float4 *>(row + 32 + 4 * j) =
+                        make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+            }
+            __syncthreads();
+            // piece q: channel half q / 3 of tap (row of taps, q % 3), or row q
+            const int col = Cin == 128 ? (dyi * 3 + q % 3) * 128 + (q / 3) * 64 : q * kN;
+            for (int e = tid; e < 128 * (kPiece / 4); e += kWgThreads) {
+                const int o = e / (kPiece / 4), c = (e - o * (kPiece / 4)) * 4;
+                const float4 f = *reinterpret_cast<const float4 *>(stg + o * kLd + c);
+                // 16-byte aligned: rows, taps and channels are multiples of four
+                atomicAdd(reinterpret_cast<float4 *>(dw + (size_t)o * (9 * Cin) + col + c), f);
+            }
+            __syncthreads();
         }
-    } else if (s_fail && tid == 0) {
+        if (warp < 4 && nbias > 0) {
+            float v[16];
+            tc::tmem_ld16(lanes + kBiasCol, v);
+            atomicAdd(db + warp * 32 + lane, v[0]);
+        }
+    } else if (sh.fail && tid == 0) {
         atomicOr(err, 1u);
-        for (int s = s_consumed; s < s_issued; ++s)
-            tc::mbar_wait_bounded(&full[s % kWStages], (s / kWStages) & 1);
+        for (int s = sh.used; s < sh.issued; ++s)
+            tc::mbar_wait_bounded(&sh.full[s % sp.stages], (s / sp.stages) & 1);
     }
     tc::fence_before_sync();
     __syncthreads();
-    if (warp == 0) tc::tmem_dealloc(tmem, 128);
+    if (warp == 4) tc::tmem_dealloc(tmem, kCols);
 }
 
 // First layer (16 -> 128 channels): one tap per 16-wide K slab.  The
@@ -805,6 +902,45 @@ StripShape conv_shape(int S, int d)
     return sp;
 }
 
+// NHWC tensor of 128 (box 64, 128-byte swizzle) or 16 channels (32-byte
+// swizzle); box w x h pixels.
+bool map_nhwc(CUtensorMap *m, const uint16_t *ptr, int ch, int n, int S, int w, int h)
+{
+    auto fn = encoder();
+    if (!fn) return false;
+    const cuuint64_t row = (cuuint64_t)ch * 2;
+    const cuuint64_t dims[4] = {(cuuint64_t)ch, (cuuint64_t)S, (cuuint64_t)S, (cuuint64_t)n};
+    const cuuint64_t strides[3] = {row, (cuuint64_t)S * row, (cuuint64_t)S * S * row};
+    const cuuint32_t box[4] = {ch == 128 ? 64u : 16u, (cuuint32_t)w, (cuuint32_t)h, 1};
+    const cuuint32_t es[4] = {1, 1, 1, 1};
+    return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<uint16_t *>(ptr), dims,
+              strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+              ch == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_32B,
+              CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// Slabs and strips of the weight gradient: 128 pixels where two stages fit,
+// else 64.
+WgradShape wgrad_shape(int S, int d, int cin)
+{
+    const int strips = cin == 128 ? 2 : 3, row = cin == 128 ? 128 : 32;
+    for (int L = 128;; L = 64) {
+        WgradShape sp{};
+        const int w = S < L ? S : L, R = L / w;
+        sp.L = L;
+        while ((1 << sp.lgw) < w) ++sp.lgw;
+        const bool one = w + 2 * d <= 256 && w + 2 * d < 3 * w;
+        sp.pitch = one ? w + 2 * d : w;
+        sp.nbox = one ? 1 : 3;
+        sp.box = R * sp.pitch * row;
+        sp.tap = one ? d * row : sp.box;
+        sp.strip = (sp.nbox * sp.box + 1023) / 1024 * 1024;
+        sp.stages = std::min(kMaxWgStages, kWgRoom / (L * 256 + strips * sp.strip));
+        if (sp.stages >= 2 || L == 64) return sp;
+    }
+}
+
 // First-layer input [n][S][S][16] BF16; box 16 channels x 128 pixels.
 bool map_in16(CUtensorMap *m, const uint16_t *ptr, int n, int S)
 {
@@ -885,31 +1021,40 @@ cudaError_t launch_conv_tma(int mode, const uint16_t *in, const uint16_t *w,
     return cudaGetLastError();
 }
 
-// CTAs of the weight-gradient kernel resident per SM.
-int wgrad_ctas_per_sm() { return convtma::kWCtasPerSm; }
-
-// Weight gradient of a 128 -> 128 layer, added into dw[128][1152] (FP32,
-// cleared by the caller): dz and in are [n][S][S][128] BF16, S a power of two
-// >= 16; the pixel range is split `split` ways.
-cudaError_t launch_wgrad_tma(const uint16_t *dz, const uint16_t *in, float *dw, int n,
-                             int S, int lgS, int d, int split, uint32_t *err,
+// Weight gradient, added into dw[128][9 cin] (FP32, cleared by the caller), and
+// bias gradient, added into db[128], of a layer of cin = 16 or 128 input
+// channels: dz [n][S][S][128] and in [n][S][S][cin] BF16, S a power of two >=
+// 16; the pixel range is split over the SMs.
+cudaError_t launch_wgrad_tma(const uint16_t *dz, const uint16_t *in, int cin, float *dw,
+                             float *db, int n, int S, int lgS, int d, uint32_t *err,
                              cudaStream_t st)
 {
     using namespace convtma;
-    if (S < 16 || (S & (S - 1)) || ((uintptr_t)dz & 15) || ((uintptr_t)in & 15) ||
-        ((uintptr_t)dw & 15) || split < 1)
+    if (S < 16 || (S & (S - 1)) || (cin != 16 && cin != 128) || ((uintptr_t)dz & 15) ||
+        ((uintptr_t)in & 15) || ((uintptr_t)dw & 15))
         return cudaErrorInvalidValue;
+    const WgradShape sp = wgrad_shape(S, d, cin);
     CUtensorMap mz, mi;
-    if (!map_act(&mz, dz, n, S, 64) || !map_act(&mi, in, n, S, 64))
+    const int w = 1 << sp.lgw;
+    if (!map_nhwc(&mz, dz, 128, n, S, w, sp.L / w) ||
+        !map_nhwc(&mi, in, cin, n, S, sp.pitch, sp.L / w))
         return cudaErrorInvalidValue;
-    cudaError_t attr = cudaFuncSetAttribute(
-        k_wgrad_tma, cudaFuncAttributeMaxDynamicSharedMemorySize, kWSmem);
+    const bool eight = sp.L == 128;
+    const auto kern = cin == 128 ? (eight ? k_wgrad_strip<128, 8> : k_wgrad_strip<128, 4>)
+                                 : (eight ? k_wgrad_strip<16, 8> : k_wgrad_strip<16, 4>);
+    int dev = 0, nsm = 0;
+    cudaError_t attr = cudaGetDevice(&dev);
+    if (attr == cudaSuccess)
+        attr = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    const int smem = 227 * 1024;
+    if (attr == cudaSuccess)
+        attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (attr != cudaSuccess) return attr;
-    const int total = (int)((long long)n * S * S / 64);
-    if (split > total) split = total;
-    const int per = (total + split - 1) / split;
-    dim3 grid(1, 9, (total + per - 1) / per);
-    k_wgrad_tma<<<grid, 128, kWSmem, st>>>(mz, mi, dw, S, lgS, d, total, per, err);
+    const int total = (int)((long long)n * S * S / sp.L);
+    const int rows = cin == 128 ? 3 : 1;   // rows of taps, one per CTA
+    const int per = (total + nsm / rows - 1) / (nsm / rows);
+    kern<<<dim3((total + per - 1) / per, rows), kWgThreads, smem, st>>>(
+        mz, mi, dw, db, S, lgS, d, sp, total, per, err);
     return cudaGetLastError();
 }
 

@@ -31,11 +31,6 @@
 #include <cmath>
 #include <cstring>
 
-namespace fire {
-// CTAs of the weight-gradient kernel resident per SM (fire_conv_tma.cu).
-int wgrad_ctas_per_sm();
-}  // namespace fire
-
 using namespace fire;
 
 namespace {
@@ -752,22 +747,25 @@ int fire_net_backward(fire_ctx *ctx, fire_net *net, int n, const uint16_t *x,
     const int kslabs = P / 64;
     for (int l = kL - 1; l >= 0; --l) {
         cudaError_t e;
-        if (l == 0) {
-            ConvWgrad<kCin> p{net->dz[0], x, net->grad + w_off(0), kC, 9 * kCin, P,
-                              S, lgS, kDil[0]};
-            e = tc::launch_tc_tile<64>(p, wgrad_split(3, kslabs), err, st);
-        } else if (S >= 16) {
-            e = launch_wgrad_tma(net->dz[l], net->h[l - 1], net->grad + w_off(l), n, S,
-                                 lgS, kDil[l],
-                                 wgrad_split(9, kslabs, wgrad_ctas_per_sm()), err, st);
+        if (S >= 16) {
+            e = launch_wgrad_tma(net->dz[l], l ? net->h[l - 1] : x, l ? kC : kCin,
+                                 net->grad + w_off(l), net->grad + b_off(l), n, S, lgS,
+                                 kDil[l], err, st);
+            CUDA_TRY(ctx, e, "weight gradient");
         } else {
-            ConvWgrad<kC> p{net->dz[l], net->h[l - 1], net->grad + w_off(l), kC,
-                            9 * kC, P, S, lgS, kDil[l]};
-            e = tc::launch_tc_tile<128>(p, wgrad_split(9, kslabs), err, st);
+            if (l == 0) {
+                ConvWgrad<kCin> p{net->dz[0], x, net->grad + w_off(0), kC, 9 * kCin, P,
+                                  S, lgS, kDil[0]};
+                e = tc::launch_tc_tile<64>(p, wgrad_split(3, kslabs), err, st);
+            } else {
+                ConvWgrad<kC> p{net->dz[l], net->h[l - 1], net->grad + w_off(l), kC,
+                                9 * kC, P, S, lgS, kDil[l]};
+                e = tc::launch_tc_tile<128>(p, wgrad_split(9, kslabs), err, st);
+            }
+            CUDA_TRY(ctx, e, "weight gradient");
+            k_bias_grad<<<nblk, 256, 0, st>>>(net->dz[l], P, per, net->grad + b_off(l));
+            CUDA_TRY(ctx, cudaGetLastError(), "bias gradient");
         }
-        CUDA_TRY(ctx, e, "weight gradient");
-        k_bias_grad<<<nblk, 256, 0, st>>>(net->dz[l], P, per, net->grad + b_off(l));
-        CUDA_TRY(ctx, cudaGetLastError(), "bias gradient");
         if (l > 0) {
             const uint16_t *wt = net->wt + (size_t)(l - 1) * kWl;
             if (S >= 16) {

@@ -80,3 +80,49 @@ def test_layers(S, n):
         hin = h
     net.free()
     ctx.close()
+
+
+@pytest.mark.parametrize("S,n", [(8, 3), (16, 1), (16, 3), (32, 2), (64, 1),
+                                 (64, 3), (128, 1), (256, 1), (512, 1)])
+def test_weight_gradients(S, n):
+    """dW and db of every layer from the device's own dz and layer input.
+
+    The pixels (P) are split over at least 50 blocks per tap, each a chain of
+    FP32 additions of 16-pixel products (at most P / 800 + 8 of them), and the
+    blocks' sums (at most 152) are added with atomics; an addition errs by at
+    most 2^-23 of what it adds up to (the tensor core truncates), which the sum
+    of absolute products bounds.
+    """
+    torch.manual_seed(S + n)
+    ctx = fire.Context(0, torch.cuda.current_stream())
+    theta = surrogate.init_params(2 * S + n, head_bias=-1.0)
+    net = fire.Net(ctx, S, n)
+    net.set_params(theta)
+    x = torch.rand((n, S, S, 16), device="cuda").to(torch.bfloat16)
+    t = torch.rand((n, S, S), device="cuda")
+    net.backward(x, t, None, sync=True)
+    grad = torch.tensor(net.get(fire.NET_GRAD), device="cuda").double()
+    eps = (n * S * S / 800 + 160) * 2.0 ** -23
+
+    def buf(which, l):
+        o = torch.empty((n, S, S, 128), dtype=torch.bfloat16, device="cuda")
+        return net.buffer(which, l, n, o).double()
+
+    off, hin = 0, x.double()
+    for l, d in enumerate(DIL):
+        ci = hin.shape[-1]
+        nw = 128 * 9 * ci
+        dz = buf(fire.BUF_DZ, l).reshape(-1, 128)
+        hp = torch.nn.functional.pad(hin, (0, 0, d, d, d, d))
+        gw = grad[off:off + nw].view(128, 9, ci)
+        for tap in range(9):
+            r, c = (tap // 3) * d, (tap % 3) * d
+            xs = hp[:, r:r + S, c:c + S, :].reshape(-1, ci)
+            want, mag = dz.T @ xs, dz.abs().T @ xs.abs()
+            assert bool(((gw[:, tap] - want).abs() <= eps * mag).all()), (l, tap)
+        gb = grad[off + nw:off + nw + 128]
+        assert bool(((gb - dz.sum(0)).abs() <= eps * dz.abs().sum(0)).all()), l
+        off += nw + 128
+        hin = buf(fire.BUF_ACT, l)
+    net.free()
+    ctx.close()
