@@ -1,7 +1,7 @@
 // TMA-fed implicit-GEMM convolutions of the surrogate network on tcgen05
 // tensor cores: the 128 -> 128 layers forward and input gradient
 // (k_conv_pair), the weight and bias gradients of all layers (k_wgrad_strip)
-// and the first layer forward (k_conv1_tma).
+// and the first layer forward (k_conv1).
 //
 // In each, one thread issues tensor-map copies of shifted NHWC activation
 // boxes (channels, x, y, sample; out-of-range elements read as zero, which is
@@ -25,11 +25,15 @@ namespace fire {
 namespace convtma {
 
 constexpr int kSlabs = 18;                      // 9 taps x 2 channel halves
+// Epilogues: forward (bias + ReLU), input gradient (ReLU mask of the layer
+// below), forward with the network's head behind it.
+constexpr int kFwd = 0, kDgrad = 1, kFwdHead = 2;
+
 struct Epi {
-    int mode;                 // 0 forward (bias + ReLU), 1 input gradient (mask)
     const float *bias;        // forward
     const uint16_t *hprev;    // input gradient: activations of the layer below
     uint16_t *out;            // [P][128] BF16
+    HeadArgs head;
 };
 
 __device__ __forceinline__ uint64_t desc_sw128(uint32_t saddr)
@@ -141,6 +145,12 @@ __device__ __forceinline__ uint32_t leader_addr(const void *p)
     return r;
 }
 
+__device__ __forceinline__ void mbar_arrive(void *bar)
+{
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_addr(bar))
+                 : "memory");
+}
+
 __device__ __forceinline__ void arrive_cluster(uint32_t cluster_addr)
 {
     asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(
@@ -227,31 +237,61 @@ constexpr int kStripRoom = 80 * 1024;
 constexpr int kMaxA = 5;
 constexpr int kEpiWarps = 4;
 constexpr int kPairThreads = 32 * (kEpiWarps + 3);
-constexpr int kPairSmem = kWBytes + kStripRoom + 2048;   // + alignment, barriers
+constexpr int kPairSmem = kWBytes + kStripRoom + 3072;   // + alignment, barriers
 
 struct PairShared {
     unsigned long long afull[kMaxA], aempty[kMaxA], wfull[kSlabs];
     unsigned long long tfull[2], tempty[2], done;
     uint32_t tmem_slot;
     int fail, issued, used;
-    float bias[128];
+    float bias[128], head[129];
 };
-static_assert(sizeof(PairShared) <= 1024, "barrier area");
+static_assert(sizeof(PairShared) <= 2048, "barrier area");
+
+__device__ __forceinline__ float bf16_lo(uint32_t u) { return __uint_as_float(u << 16); }
+__device__ __forceinline__ float bf16_hi(uint32_t u)
+{
+    return __uint_as_float(u & 0xffff0000u);
+}
+
+// Probability, gradient and loss term of pixel p from the head's 16 partial
+// sums of eight channels each (added in the order of k_head, whose 16 lanes
+// hold one each).
+__device__ __forceinline__ void head_pixel(const HeadArgs &hd, float bias,
+                                           const float part[16], size_t p)
+{
+    float v[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = part[i] + part[i + 8];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) v[i] += v[i + 4];
+    const float z = ((v[0] + v[2]) + (v[1] + v[3])) + bias;
+    const float y = 1.0f / (1.0f + expf(-z));
+    hd.prob[p] = y;
+    if (hd.target) {
+        const float t = hd.target[p];
+        hd.term[p] = fmaxf(z, 0.0f) - t * z + log1pf(expf(-fabsf(z)));
+        hd.g[p] = (y - t) * hd.inv_count;
+    }
+}
 
 // Epilogue of one accumulator row (pixel p, 128 channels in tensor memory at
 // taddr): forward, bias and ReLU; input gradient, zero where the layer
-// below's activation (mask) is not positive; BF16 stores.
+// below's activation (mask) is not positive; BF16 stores.  s_head: the head's
+// weights and bias.
+template <int kMode>
 __device__ __forceinline__ void pair_epilogue(const Epi &epi, const float *s_bias,
-                                              uint32_t taddr, size_t p,
-                                              const uint32_t mask[64])
+                                              const float *s_head, uint32_t taddr,
+                                              size_t p, const uint32_t *mask)
 {
     uint16_t *orow = epi.out + p * 128;
+    float part[16];
 #pragma unroll
     for (int c0 = 0; c0 < 128; c0 += 32) {
         float v[32];
         tc::tmem_ld32(taddr + (uint32_t)c0, v);
         uint32_t pk[16];
-        if (epi.mode == 0) {
+        if (kMode != kDgrad) {
 #pragma unroll
             for (int j = 0; j < 16; ++j)
                 pk[j] = pack2(fmaxf(v[2 * j] + s_bias[c0 + 2 * j], 0.0f),
@@ -264,9 +304,22 @@ __device__ __forceinline__ void pair_epilogue(const Epi &epi, const float *s_bia
                               pos16(h >> 16) ? v[2 * j + 1] : 0.0f);
             }
         }
+        if (kMode == kFwdHead) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                float z = 0.0f;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    z = fmaf(bf16_lo(pk[4 * q + j]), s_head[c0 + 8 * q + 2 * j], z);
+                    z = fmaf(bf16_hi(pk[4 * q + j]), s_head[c0 + 8 * q + 2 * j + 1], z);
+                }
+                part[c0 / 8 + q] = z;
+            }
+        }
         st_global32(orow + c0, pk);
         st_global32(orow + c0 + 16, pk + 8);
     }
+    if (kMode == kFwdHead) head_pixel(epi.head, s_head[128], part, p);
 }
 
 // Convolution of a 128 -> 128 layer on CTA pairs (cta_group::2).  The pair
@@ -299,7 +352,7 @@ __device__ __forceinline__ void pair_epilogue(const Epi &epi, const float *s_bia
 //
 // sign = +1: forward (source pixel p + off(t)); -1: input gradient (p - off(t)).
 // A strip of `px` pixels serves kTaps taps (StripShape); `na` strip stages.
-template <int kTaps>
+template <int kTaps, int kMode>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
     k_conv_pair(const __grid_constant__ CUtensorMap act,
                 const __grid_constant__ CUtensorMap wts, Epi epi, int px, int na, int S,
@@ -315,7 +368,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int rank = (int)cluster_rank();
     const int pair0 = blockIdx.x >> 1, pstep = gridDim.x >> 1;
-    if (epi.mode == 0 && tid < 128) sh.bias[tid] = epi.bias[tid];
+    if (kMode != kDgrad && tid < 128) sh.bias[tid] = epi.bias[tid];
+    if (kMode == kFwdHead && tid <= 128) sh.head[tid] = epi.head.wh[tid];
     if (warp == kEpiWarps) tmem_alloc_pair(&sh.tmem_slot, 256);
     if (tid == 0) {
         for (int i = 0; i < kMaxA; ++i) {
@@ -457,7 +511,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
             const int acc = it & 1;
             const size_t p = (size_t)(2 * pr + rank) * 128 + warp * 32 + lane;
             uint32_t mask[64];
-            if (epi.mode != 0) {
+            if (kMode == kDgrad) {
 #pragma unroll
                 for (int j = 0; j < 8; ++j)
                     ld_global32(epi.hprev + p * 128 + 16 * j, mask + 8 * j);
@@ -468,9 +522,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
                 break;
             }
             tc::fence_after_sync();
-            pair_epilogue(epi, sh.bias,
-                          tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(acc * 128), p,
-                          mask);
+            pair_epilogue<kMode>(epi, sh.bias, sh.head,
+                                 tmem + ((uint32_t)(warp * 32) << 16) +
+                                     (uint32_t)(acc * 128),
+                                 p, mask);
             tc::fence_before_sync();
             __syncwarp();
             if (lane == 0) arrive_cluster(leader_addr(&sh.tempty[acc]));
@@ -732,16 +787,26 @@ __global__ void __launch_bounds__(kWgThreads, 1)
     if (warp == 4) tc::tmem_dealloc(tmem, kCols);
 }
 
-// First layer (16 -> 128 channels): one tap per 16-wide K slab.  The
-// activation box is 16 channels (32 bytes) x 128 pixels and the weight box
-// 16 x 128 rows of W1[o][t][i]; both land 32-byte swizzled, the canonical
-// K-major SWIZZLE_32B layout (8-row groups 256 bytes apart), and one
-// 128 x 128 x 16 MMA consumes a slab.  Nine slabs, no padding of K.
-constexpr int kC1Stages = 6;                     // 49 KB: four CTAs per SM, as
-                                                  // many as tensor memory holds
+// First layer (16 -> 128 channels): K = 9 taps x 16 channels, one 128 x 128 x
+// 16 MMA per tap, in tap order; rows of 32 bytes, 32-byte swizzle.  Bound by
+// writing the activations (134 MB at 8 x 256 x 256, 20 us of fallback copy
+// bandwidth), so the kernel is built around its epilogue: one persistent CTA
+// per SM, the weights loaded once, four tensor-memory accumulators, two groups
+// of four epilogue warps on alternate tiles.  A tile's input is three strips
+// of 130 pixels, one per row of taps (S >= 128), or nine boxes, one per tap.
+// 37.6 us; one tile per CTA, four to an SM, spent its time setting up: 95 us.
 constexpr int kC1Tile = 128 * 32;                 // 128 rows x 16 BF16
-constexpr int kC1Stage = 2 * kC1Tile;
-constexpr int kC1Smem = kC1Stages * kC1Stage + 1024;
+constexpr int kC1Threads = 320;
+constexpr int kC1Stages = 4;
+
+struct C1Shared {
+    unsigned long long full[kC1Stages], empty[kC1Stages], wfull;
+    unsigned long long tfull[4], tempty[4], done;
+    uint32_t tmem_slot;
+    int fail, issued, used;
+    float bias[128];
+};
+static_assert(sizeof(C1Shared) <= 1024, "barrier area");
 
 __device__ __forceinline__ uint64_t desc_sw32(uint32_t saddr)
 {
@@ -753,108 +818,150 @@ __device__ __forceinline__ uint64_t desc_sw32(uint32_t saddr)
     return d;
 }
 
-__global__ void __launch_bounds__(128, 4)
-    k_conv1_tma(const __grid_constant__ CUtensorMap act,
-                const __grid_constant__ CUtensorMap wts, const float *bias,
-                uint16_t *out, int S, int lgS, uint32_t *err)
+// kBoxes: 3 strips of 130 pixels (5 KB apart) or 9 boxes of 128 (4 KB).
+template <int kBoxes>
+__global__ void __launch_bounds__(kC1Threads, 1)
+    k_conv1(const __grid_constant__ CUtensorMap act,
+            const __grid_constant__ CUtensorMap wts, Epi epi, int S, int lgS, int ntiles,
+            uint32_t *err)
 {
+    constexpr uint32_t kBoxStep = kBoxes == 3 ? 5120 : kC1Tile;
+    constexpr uint32_t kBoxTx = kBoxes == 3 ? 130 * 32 : kC1Tile;
+    constexpr uint32_t kStage = kBoxes * kBoxStep;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
-    __shared__ __align__(8) unsigned long long full[kC1Stages], empty[kC1Stages], done;
-    __shared__ uint32_t tmem_slot;
-    __shared__ int s_fail, s_issued, s_consumed;
-    __shared__ float s_bias[128];
+    const uint32_t raw = tc::smem_addr(smem_raw);
+    const uint32_t base = (raw + 1023u) & ~1023u;
+    const uint32_t wbase = base + kC1Stages * kStage;
+    C1Shared &sh = *reinterpret_cast<C1Shared *>(smem_raw + (base - raw) +
+                                                 kC1Stages * kStage + 9 * kC1Tile);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const uint32_t base = (tc::smem_addr(smem_raw) + 1023u) & ~1023u;
-    const int m0 = blockIdx.x * 128;
-    const int b = m0 >> (2 * lgS);
-    const int y0 = (m0 >> lgS) & (S - 1), x0 = m0 & (S - 1);
-    s_bias[tid] = bias[tid];
-
-    if (warp == 0) {
-        tc::tmem_alloc(&tmem_slot, 128);
+    if (tid < 128) sh.bias[tid] = epi.bias[tid];
+    if (warp == 8) {
+        tc::tmem_alloc(&sh.tmem_slot, 512);
         tc::tmem_relinquish();
     }
     if (tid == 0) {
         for (int i = 0; i < kC1Stages; ++i) {
-            tc::mbar_init(&full[i], 1);
-            tc::mbar_init(&empty[i], 1);
+            tc::mbar_init(&sh.full[i], 1);
+            tc::mbar_init(&sh.empty[i], 1);
         }
-        tc::mbar_init(&done, 1);
-        s_fail = 0;
-        s_issued = 0;
-        s_consumed = 0;
+        tc::mbar_init(&sh.wfull, 1);
+        for (int i = 0; i < 4; ++i) {
+            tc::mbar_init(&sh.tfull[i], 1);
+            tc::mbar_init(&sh.tempty[i], 4);
+        }
+        tc::mbar_init(&sh.done, 1);
+        sh.fail = sh.issued = sh.used = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
-    const uint32_t tmem = tmem_slot;
+    const uint32_t tmem = sh.tmem_slot;
 
-    if (warp == 0 && lane == 0) {
-        int s = 0;
-        for (; s < 9; ++s) {
-            const int st = s % kC1Stages;
-            if (s >= kC1Stages &&
-                !tc::mbar_wait_bounded(&empty[st], ((s / kC1Stages) - 1) & 1)) {
-                atomicOr(&s_fail, 1);
-                break;
-            }
-            if (*(volatile int *)&s_fail) break;
-            const int dy = s / 3 - 1, dx = s % 3 - 1;   // dilation 1
-            const uint32_t sa = base + st * kC1Stage;
-            expect_tx(&full[st], kC1Stage);
-            tma_4d(sa, &act, 0, x0 + dx, y0 + dy, b, &full[st]);
-            tma_2d(sa + kC1Tile, &wts, s * 16, 0, &full[st]);
+    if (warp == 8) {
+        // loader
+        const bool leader = elect_one();
+        if (leader) {
+            expect_tx(&sh.wfull, 9 * kC1Tile);
+            for (int t = 0; t < 9; ++t)
+                tma_2d(wbase + t * kC1Tile, &wts, t * 16, 0, &sh.wfull);
         }
-        s_issued = s;
-    } else if (warp == 1 && lane == 0) {
+        __syncwarp();
+        int g = 0;
+        bool ok = true;
+        for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++g) {
+            const int st = g % kC1Stages;
+            if (g >= kC1Stages)
+                ok = all_ok(tc::mbar_wait_bounded(&sh.empty[st], ((g / kC1Stages) - 1) & 1));
+            ok = all_ok(ok && !*(volatile int *)&sh.fail);
+            if (!ok) break;
+            if (leader) {
+                const int m0 = tile * 128;
+                const int b = m0 >> (2 * lgS);
+                const int y = (m0 >> lgS) & (S - 1), x = m0 & (S - 1);
+                const uint32_t sa = base + st * kStage;
+                expect_tx(&sh.full[st], kBoxes * kBoxTx);
+                for (int i = 0; i < kBoxes; ++i)
+                    tma_4d(sa + i * kBoxStep, &act, 0,
+                           x + (kBoxes == 3 ? -1 : i % 3 - 1),
+                           y + (kBoxes == 3 ? i - 1 : i / 3 - 1), b, &sh.full[st]);
+            }
+            __syncwarp();
+        }
+        if (leader) {
+            if (!ok) atomicOr(&sh.fail, 1);
+            sh.issued = g;
+        }
+        __syncwarp();
+    } else if (warp == 9) {
+        // MMA issuer: tile number g of this CTA accumulates in buffer g mod 4
         constexpr uint32_t idesc = tc::idesc_bf16(128, 128);
-        int s = 0;
-        for (; s < 9; ++s) {
-            const int st = s % kC1Stages;
-            if (!tc::mbar_wait_bounded(&full[st], (s / kC1Stages) & 1)) {
-                atomicOr(&s_fail, 1);
+        const uint64_t ad = desc_sw32(base), wd = desc_sw32(wbase);
+        const bool leader = elect_one();
+        int g = 0;
+        bool ok = all_ok(tc::mbar_wait_bounded(&sh.wfull, 0));
+        for (int tile = blockIdx.x; ok && tile < ntiles; tile += gridDim.x, ++g) {
+            const int st = g % kC1Stages, acc = g & 3;
+            if (g >= 4) ok = all_ok(tc::mbar_wait_bounded(&sh.tempty[acc], ((g >> 2) - 1) & 1));
+            ok = ok && all_ok(tc::mbar_wait_bounded(&sh.full[st], (g / kC1Stages) & 1));
+            if (!ok) break;
+            tc::fence_after_sync();
+            const uint64_t a0 = ad + st * (kStage >> 4);
+            if (leader) {
+#pragma unroll
+                for (int t = 0; t < 9; ++t)
+                    tc::mma_bf16(tmem + acc * 128,
+                                 a0 + (kBoxes == 3 ? (t / 3) * (kBoxStep >> 4) + (t % 3) * 2
+                                                   : t * (kBoxStep >> 4)),
+                                 wd + t * (kC1Tile >> 4), idesc, t > 0);
+                tc::mma_commit(&sh.empty[st]);
+                tc::mma_commit(&sh.tfull[acc]);
+            }
+            __syncwarp();
+        }
+        if (leader) {
+            if (!ok) atomicOr(&sh.fail, 1);
+            sh.used = g;
+            tc::mma_commit(&sh.done);   // arrives once every issued MMA is done
+        }
+        __syncwarp();
+    } else {
+        // epilogue: warps 0..3 the even tiles of this CTA, 4..7 the odd ones
+        const int q = warp & 3;
+        for (int g = warp >> 2, tile = blockIdx.x + (warp >> 2) * gridDim.x; tile < ntiles;
+             g += 2, tile += 2 * gridDim.x) {
+            const int acc = g & 3;
+            if (*(volatile int *)&sh.fail ||
+                !tc::mbar_wait_bounded(&sh.tfull[acc], (g >> 2) & 1)) {
+                atomicOr(&sh.fail, 1);
                 break;
             }
             tc::fence_after_sync();
-            const uint32_t sa = base + st * kC1Stage;
-            tc::mma_bf16(tmem, desc_sw32(sa), desc_sw32(sa + kC1Tile), idesc, s > 0);
-            tc::mma_commit(&empty[st]);
+            pair_epilogue<kFwd>(epi, sh.bias, nullptr,
+                                tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * 128),
+                                (size_t)tile * 128 + q * 32 + lane, nullptr);
+            tc::fence_before_sync();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sh.tempty[acc]);
         }
-        s_consumed = s;
-        if (s == 9) tc::mma_commit(&done);
     }
-    __syncwarp();
-    if (!tc::mbar_wait_bounded(&done, 0)) atomicOr(&s_fail, 1);
     __syncthreads();
-    tc::fence_after_sync();
-
-    if (!s_fail) {
-        const int p = m0 + warp * 32 + lane;
-        uint16_t *orow = out + (size_t)p * 128;
-#pragma unroll 1
-        for (int c0 = 0; c0 < 128; c0 += 32) {
-            float v[32];
-            tc::tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
-            uint32_t pk[16];
-#pragma unroll
-            for (int j = 0; j < 16; ++j)
-                pk[j] = pack2(fmaxf(v[2 * j] + s_bias[c0 + 2 * j], 0.0f),
-                              fmaxf(v[2 * j + 1] + s_bias[c0 + 2 * j + 1], 0.0f));
-            uint4 *o = reinterpret_cast<uint4 *>(orow + c0);
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-                o[q] = make_uint4(pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
+    if (tid == 0) {
+        if (sh.fail) {
+            atomicOr(err, 1u);
+            // copies issued but never consumed must land before the CTA leaves
+            tc::mbar_wait_bounded(&sh.wfull, 0);
+            for (int g = sh.used; g < sh.issued; ++g)
+                tc::mbar_wait_bounded(&sh.full[g % kC1Stages], (g / kC1Stages) & 1);
         }
-    } else if (tid == 0) {
-        atomicOr(err, 1u);
-        for (int s = s_consumed; s < s_issued; ++s)
-            tc::mbar_wait_bounded(&full[s % kC1Stages], (s / kC1Stages) & 1);
+        tc::mbar_wait_bounded(&sh.done, 0);
     }
     tc::fence_before_sync();
     __syncthreads();
-    if (warp == 0) tc::tmem_dealloc(tmem, 128);
+    tc::fence_after_sync();
+    if (warp == 8) tc::tmem_dealloc(tmem, 512);
 }
 
 // --- host: tensor maps ------------------------------------------------------
@@ -941,22 +1048,6 @@ WgradShape wgrad_shape(int S, int d, int cin)
     }
 }
 
-// First-layer input [n][S][S][16] BF16; box 16 channels x 128 pixels.
-bool map_in16(CUtensorMap *m, const uint16_t *ptr, int n, int S)
-{
-    auto fn = encoder();
-    if (!fn) return false;
-    const cuuint64_t dims[4] = {16, (cuuint64_t)S, (cuuint64_t)S, (cuuint64_t)n};
-    const cuuint64_t strides[3] = {32, (cuuint64_t)S * 32, (cuuint64_t)S * S * 32};
-    const cuuint32_t bx = S >= 128 ? 128 : S, by = 128 / bx;
-    const cuuint32_t box[4] = {16, bx, by, 1};
-    const cuuint32_t es[4] = {1, 1, 1, 1};
-    return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<uint16_t *>(ptr), dims,
-              strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_32B,
-              CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 // First-layer weights [128 rows][144] BF16; box 16 x 128.
 bool map_w144(CUtensorMap *m, const uint16_t *ptr)
 {
@@ -991,12 +1082,13 @@ bool map_wts(CUtensorMap *m, const uint16_t *ptr)
 
 // Forward (mode 0: out = ReLU(conv(in) + bias)) or input gradient (mode 1:
 // out = conv^T(in) masked by hprev > 0) of a 128 -> 128 layer over n samples
+// (head: forward only, the network's head on the result)
 // of S x S (S a power of two >= 16).  `w` is W[o][t][i] (forward) or
 // Wt[i][t][o] (input gradient), 16-byte aligned.
 cudaError_t launch_conv_tma(int mode, const uint16_t *in, const uint16_t *w,
                             const float *bias, const uint16_t *hprev, uint16_t *out,
-                            int n, int S, int lgS, int d, uint32_t *err,
-                            cudaStream_t st)
+                            int n, int S, int lgS, int d, const HeadArgs *head,
+                            uint32_t *err, cudaStream_t st)
 {
     using namespace convtma;
     if (S < 16 || (S & (S - 1)) || ((uintptr_t)in & 15) || ((uintptr_t)w & 15))
@@ -1004,12 +1096,16 @@ cudaError_t launch_conv_tma(int mode, const uint16_t *in, const uint16_t *w,
     const StripShape sp = conv_shape(S, d);
     CUtensorMap ma, mw;
     if (!map_act(&ma, in, n, S, sp.px) || !map_wts(&mw, w)) return cudaErrorInvalidValue;
-    Epi e{mode, bias, hprev, out};
+    Epi e{bias, hprev, out, head ? *head : HeadArgs{}};
     int dev = 0, nsm = 0;
     cudaError_t attr = cudaGetDevice(&dev);
     if (attr == cudaSuccess)
         attr = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    const auto kern = sp.taps == 3 ? k_conv_pair<3> : k_conv_pair<1>;
+    const bool three = sp.taps == 3;
+    const auto kern =
+        mode != 0 ? (three ? k_conv_pair<3, kDgrad> : k_conv_pair<1, kDgrad>)
+        : head    ? (three ? k_conv_pair<3, kFwdHead> : k_conv_pair<1, kFwdHead>)
+                  : (three ? k_conv_pair<3, kFwd> : k_conv_pair<1, kFwd>);
     if (attr == cudaSuccess)
         attr = cudaFuncSetAttribute(
             kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kPairSmem);
@@ -1068,13 +1164,22 @@ cudaError_t launch_conv1_tma(const uint16_t *x, const uint16_t *w, const float *
     if (S < 16 || (S & (S - 1)) || ((uintptr_t)x & 15) || ((uintptr_t)w & 15))
         return cudaErrorInvalidValue;
     CUtensorMap ma, mw;
-    if (!map_in16(&ma, x, n, S) || !map_w144(&mw, w)) return cudaErrorInvalidValue;
-    cudaError_t attr = cudaFuncSetAttribute(
-        k_conv1_tma, cudaFuncAttributeMaxDynamicSharedMemorySize, kC1Smem);
+    const bool strips = S >= 128;   // a tile lies in one row
+    const int bw = strips ? 130 : (S < 128 ? S : 128);
+    if (!map_nhwc(&ma, x, 16, n, S, bw, strips ? 1 : 128 / bw) || !map_w144(&mw, w))
+        return cudaErrorInvalidValue;
+    Epi e{bias, nullptr, out, HeadArgs{}};
+    const auto kern = strips ? k_conv1<3> : k_conv1<9>;
+    const int smem = kC1Stages * (strips ? 3 * 5120 : 9 * kC1Tile) + 9 * kC1Tile + 2048;
+    int dev = 0, nsm = 0;
+    cudaError_t attr = cudaGetDevice(&dev);
+    if (attr == cudaSuccess)
+        attr = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    if (attr == cudaSuccess)
+        attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (attr != cudaSuccess) return attr;
-    const long long P = (long long)n * S * S;
-    k_conv1_tma<<<(unsigned)(P / 128), 128, kC1Smem, st>>>(ma, mw, bias, out, S, lgS,
-                                                           err);
+    const int ntiles = (int)((long long)n * S * S / 128);
+    kern<<<std::min(ntiles, nsm), kC1Threads, smem, st>>>(ma, mw, e, S, lgS, ntiles, err);
     return cudaGetLastError();
 }
 

@@ -271,10 +271,19 @@ int noalloc_take_error(int device, bool *set);
 // grown, so a state that fits in shared memory goes there).
 int plan_launch(fire_ctx *ctx, int ntiles, long long n, LaunchPlan *p,
                 bool burn = false, bool fixed_scratch = false);
+// The network's head on the top layer's activations: probabilities, and with
+// target the per-pixel gradient g and the loss terms (summed by k_loss_sum).
+struct HeadArgs {
+    const float *wh;       // w[128], then the bias
+    float *prob;
+    const float *target;   // nullable
+    float inv_count;
+    float *g, *term;
+};
 cudaError_t launch_conv_tma(int mode, const uint16_t *in, const uint16_t *w,
                             const float *bias, const uint16_t *hprev, uint16_t *out,
-                            int n, int S, int lgS, int d, uint32_t *err,
-                            cudaStream_t st);
+                            int n, int S, int lgS, int d, const HeadArgs *head,
+                            uint32_t *err, cudaStream_t st);
 cudaError_t launch_conv1_tma(const uint16_t *x, const uint16_t *w, const float *bias,
                              uint16_t *out, int n, int S, int lgS, uint32_t *err,
                              cudaStream_t st);

@@ -28,6 +28,7 @@
 
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 
@@ -231,6 +232,32 @@ __global__ void __launch_bounds__(256)
     }
 }
 
+// Loss from the per-pixel terms of the fused head, in the groups of k_head:
+// warp w of its grid adds the pixels 2 (w + i nw) and 2 (w + i nw) + 1 for i =
+// 0, 1, ... in single precision, then the two sums; one thread per warp here.
+__global__ void __launch_bounds__(256)
+    k_loss_sum(const float2 *__restrict__ term, int P, int nw, float inv_count,
+               double *__restrict__ loss)
+{
+    const int w = blockIdx.x * blockDim.x + threadIdx.x;
+    float l0 = 0.0f, l1 = 0.0f;
+    if (w < nw)
+        for (int pp = w; 2 * pp < P; pp += nw) {
+            const float2 t = term[pp];
+            l0 += t.x * inv_count;
+            l1 += t.y * inv_count;
+        }
+    double l = (double)(l0 + l1);
+    for (int o = 16; o; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+    __shared__ double red[8];
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = l;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int i = 1; i < 8; ++i) l += red[i];
+        atomicAdd(loss, l);
+    }
+}
+
 // dz of the top layer, head weight and bias gradients.  Block = 128 threads,
 // thread c = channel; each block walks `per` pixels.
 // Head gradient: dz[p, c] = g[p] wh[c] where h[p, c] > 0 (else 0), dwh[c] =
@@ -393,26 +420,48 @@ __global__ void k_planes(int H, int W, int S, const uint8_t *__restrict__ veg,
     o[9] = cw * inv;
 }
 
-__global__ void k_inputs(int S, int H, int W, int n, const float *__restrict__ planes,
-                         const fire_params *__restrict__ params,
-                         const fire_cell *__restrict__ ign, uint16_t *__restrict__ x)
+// A thread packs its coarse cell's planes once and writes it for up to
+// kInputSamples samples, whose parameters (a double division each) and
+// ignition cells the block computes once: with both per pixel and sample the
+// divisions took 87 us for 16 x 256 x 256, whose output is 34 MB.
+constexpr int kInputSamples = 8;
+
+__global__ void __launch_bounds__(256)
+    k_inputs(int S, int H, int W, int n, const float *__restrict__ planes,
+             const fire_params *__restrict__ params,
+             const fire_cell *__restrict__ ign, uint16_t *__restrict__ x)
 {
-    const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (t >= (long long)n * S * S) return;
-    const int s = (int)(t / ((long long)S * S));
-    const int c = (int)(t - (long long)s * S * S);
-    const int ci = c / S, cj = c % S;
+    __shared__ float par[kInputSamples][5];
+    __shared__ int cell[kInputSamples];
+    const int s0 = blockIdx.y * kInputSamples, ns = min(kInputSamples, n - s0);
+    const int SS = S * S, c = blockIdx.x * blockDim.x + threadIdx.x;
+    if (threadIdx.x < 5 * ns) {
+        const int s = threadIdx.x / 5, j = threadIdx.x - 5 * s;
+        par[s][j] = (float)(params[s0 + s].b[j] / 10.0);
+    }
+    if (threadIdx.x >= 64 && threadIdx.x < 64 + ns) {
+        const fire_cell g = ign[s0 + threadIdx.x - 64];
+        // a cell outside the grid lies in no coarse cell
+        const int ci = g.row / (H / S), cj = g.col / (W / S);
+        cell[threadIdx.x - 64] =
+            ci >= 0 && ci < S && cj >= 0 && cj < S ? ci * S + cj : -1;
+    }
+    __syncthreads();
+    if (c >= SS) return;
     const float *pl = planes + (size_t)c * 10;
-    float v[16];
+    float v[10];
+#pragma unroll
     for (int k = 0; k < 10; ++k) v[k] = pl[k];
-    const fire_cell g = ign[s];
-    v[10] = (g.row / (H / S) == ci && g.col / (W / S) == cj) ? 1.0f : 0.0f;
-    for (int j = 0; j < 5; ++j) v[11 + j] = (float)(params[s].b[j] / 10.0);
-    uint32_t pk[8];
-    for (int j = 0; j < 8; ++j) pk[j] = pack_bf16x2(v[2 * j], v[2 * j + 1]);
-    uint4 *o = reinterpret_cast<uint4 *>(x + (size_t)t * kCin);
-    o[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-    o[1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+    uint32_t pk[5];
+#pragma unroll
+    for (int j = 0; j < 5; ++j) pk[j] = pack_bf16x2(v[2 * j], v[2 * j + 1]);
+    for (int s = 0; s < ns; ++s) {
+        const float *q = par[s];
+        uint4 *o = reinterpret_cast<uint4 *>(x + ((size_t)(s0 + s) * SS + c) * kCin);
+        o[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+        o[1] = make_uint4(pk[4], pack_bf16x2(cell[s] == c ? 1.0f : 0.0f, q[0]),
+                          pack_bf16x2(q[1], q[2]), pack_bf16x2(q[3], q[4]));
+    }
 }
 
 // Burn fractions per coarse cell from tile-major burnt words (reps per group).
@@ -457,35 +506,60 @@ __global__ void k_expand(int n, int reps, const fire_params *__restrict__ gp,
 }
 
 // --- screening --------------------------------------------------------------
-// Predicted Eq. 2 fitness with expected set sizes; one block per candidate.
-__global__ void k_pred_fitness(int SS, const float *__restrict__ prob,
-                               const float *__restrict__ tfrac, double cells,
-                               int kind, double *__restrict__ pred)
+// Predicted Eq. 2 fitness with expected set sizes; a cluster of kSpread blocks
+// per candidate, whose partial sums meet in the first block's shared memory.
+// Bound by double-precision additions (five a cell at about two a clock and
+// SM): 35 us for 16 x 256 x 256, where one block per candidate, on 16 SMs, took
+// 149.
+template <int kSpread>
+__global__ void __launch_bounds__(256)
+    k_pred_fitness(int SS, const float *__restrict__ prob,
+                   const float *__restrict__ tfrac, double cells, int kind,
+                   double *__restrict__ pred)
 {
-    const float *q = prob + (size_t)blockIdx.x * SS;
+    const int s = blockIdx.x / kSpread, part = blockIdx.x % kSpread;
+    const float *q = prob + (size_t)s * SS;
     double sq = 0.0, sqt = 0.0, st = 0.0;
-    for (int c = threadIdx.x; c < SS; c += blockDim.x) {
+    for (int c = part * blockDim.x + threadIdx.x; c < SS; c += kSpread * blockDim.x) {
         const double qc = q[c], tc_ = tfrac[c];
         sq += qc;
         sqt += qc * tc_;
         st += tc_;
     }
-    __shared__ double red[3][256];
-    red[0][threadIdx.x] = sq;
-    red[1][threadIdx.x] = sqt;
-    red[2][threadIdx.x] = st;
-    __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s)
-            for (int k = 0; k < 3; ++k) red[k][threadIdx.x] += red[k][threadIdx.x + s];
-        __syncthreads();
+    for (int o = 16; o; o >>= 1) {
+        sq += __shfl_xor_sync(0xffffffffu, sq, o);
+        sqt += __shfl_xor_sync(0xffffffffu, sqt, o);
+        st += __shfl_xor_sync(0xffffffffu, st, o);
     }
-    if (threadIdx.x == 0) {
-        const double sim = cells * red[0][0], inter = cells * red[1][0];
-        const double tgt = cells * red[2][0];
+    __shared__ double red[3][8 * kSpread];
+    if ((threadIdx.x & 31) == 0) {
+        const int w = part * 8 + (threadIdx.x >> 5);
+        double *r = &red[0][w];
+        if (kSpread > 1) {
+            uint64_t g;
+            asm volatile("mapa.u64 %0, %1, 0;" : "=l"(g) : "l"(r));
+            r = reinterpret_cast<double *>(g);
+        }
+        r[0] = sq;
+        r[8 * kSpread] = sqt;
+        r[16 * kSpread] = st;
+    }
+    if (kSpread > 1)
+        asm volatile("barrier.cluster.arrive.release.aligned;\n\t"
+                     "barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    else
+        __syncthreads();
+    if (part == 0 && threadIdx.x == 0) {
+        sq = sqt = st = 0.0;
+        for (int i = 0; i < 8 * kSpread; ++i) {
+            sq += red[0][i];
+            sqt += red[1][i];
+            st += red[2][i];
+        }
+        const double sim = cells * sq, inter = cells * sqt, tgt = cells * st;
         const double num = sim + tgt - 2.0 * inter;
         const double den = kind == 0 ? tgt : sim + tgt - inter;
-        pred[blockIdx.x] = num / den;
+        pred[s] = num / den;
     }
 }
 
@@ -520,7 +594,7 @@ struct fire_net {
     uint16_t *wb = nullptr, *wt = nullptr;
     uint16_t *h[kL] = {};
     uint16_t *dz[kL] = {};
-    float *prob = nullptr, *g = nullptr;
+    float *prob = nullptr, *g = nullptr, *term = nullptr;
     double *loss = nullptr;
     int step = 0;
 };
@@ -539,12 +613,17 @@ int ilog2(int v)
     return l;
 }
 
-// Forward over n <= max_batch samples of x; activations stay in net->h.
-cudaError_t net_forward(fire_net *net, int n, const uint16_t *x, uint32_t *err,
-                        cudaStream_t st)
+// Forward over n <= max_batch samples of x: probabilities into prob, and with
+// target the loss (net->loss, cleared by the caller) and the per-pixel
+// gradient (net->g); activations stay in net->h.
+cudaError_t net_forward(fire_net *net, int n, const uint16_t *x, float *prob,
+                        const float *target, uint32_t *err, cudaStream_t st)
 {
     const int S = net->S, lgS = net->lgS;
     const int M = n * S * S;
+    const float inv_count = 1.0f / (float)M;
+    const int head_blocks = (M + 255) / 256;
+    const HeadArgs head{net->theta + kHead, prob, target, inv_count, net->g, net->term};
     cudaError_t e;
     if (S >= 16) {
         e = launch_conv1_tma(x, net->wb + w_off(0), net->theta + b_off(0), net->h[0],
@@ -560,7 +639,7 @@ cudaError_t net_forward(fire_net *net, int n, const uint16_t *x, uint32_t *err,
         if (S >= 16) {
             e = launch_conv_tma(0, net->h[l - 1], net->wb + w_off(l),
                                 net->theta + b_off(l), nullptr, net->h[l], n, S, lgS,
-                                kDil[l], err, st);
+                                kDil[l], l == kL - 1 ? &head : nullptr, err, st);
         } else {
             ConvFwd<kC> p{net->h[l - 1], net->wb + w_off(l), net->theta + b_off(l),
                           net->h[l], M, kC, 9 * kC, S, lgS, kDil[l]};
@@ -568,7 +647,15 @@ cudaError_t net_forward(fire_net *net, int n, const uint16_t *x, uint32_t *err,
         }
         if (e != cudaSuccess) return e;
     }
-    return cudaSuccess;
+    if (S < 16) {
+        k_head<<<head_blocks, 256, 0, st>>>(net->h[kL - 1], net->theta + kHead, M, target,
+                                            inv_count, prob, net->g, net->loss);
+    } else if (target) {
+        const int nw = head_blocks * 8;
+        k_loss_sum<<<(nw + 255) / 256, 256, 0, st>>>(
+            reinterpret_cast<const float2 *>(net->term), M, nw, inv_count, net->loss);
+    }
+    return cudaGetLastError();
 }
 
 int wgrad_split(int nt_n, int kslabs, int ctas_per_sm = 3)
@@ -613,7 +700,8 @@ int fire_net_create(fire_ctx *ctx, int S, int max_batch, fire_net **out)
     size_t o_h[kL], o_dz[kL];
     for (int l = 0; l < kL; ++l) o_h[l] = take(pix * kC * 2);
     for (int l = 0; l < kL; ++l) o_dz[l] = take(pix * kC * 2);
-    const size_t o_prob = take(pix * 4), o_g = take(pix * 4), o_loss = take(8);
+    const size_t o_prob = take(pix * 4), o_g = take(pix * 4), o_term = take(pix * 4),
+                 o_loss = take(8);
     cudaError_t e = cudaMalloc(&net->mem, off);
     if (e != cudaSuccess) {
         delete net;
@@ -632,6 +720,7 @@ int fire_net_create(fire_ctx *ctx, int S, int max_batch, fire_net **out)
     }
     net->prob = (float *)(b + o_prob);
     net->g = (float *)(b + o_g);
+    net->term = (float *)(b + o_term);
     net->loss = (double *)(b + o_loss);
     e = cudaMemsetAsync(net->mem, 0, o_h[0], ctx->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
@@ -707,12 +796,8 @@ int fire_net_forward(fire_ctx *ctx, fire_net *net, int n, const uint16_t *x,
     for (int s0 = 0; s0 < n; s0 += net->max_batch) {
         const int nb = n - s0 < net->max_batch ? n - s0 : net->max_batch;
         CUDA_TRY(ctx, net_forward(net, nb, x + (size_t)s0 * SS * kCin,
-                                  ctx->counter + 1, ctx->stream), "surrogate forward");
-        const int P = nb * SS;
-        k_head<<<(P + 255) / 256, 256, 0, ctx->stream>>>(
-            net->h[kL - 1], net->theta + kHead, P, nullptr, 0.0f,
-            prob + (size_t)s0 * SS, nullptr, nullptr);
-        CUDA_TRY(ctx, cudaGetLastError(), "surrogate head");
+                                  prob + (size_t)s0 * SS, nullptr, ctx->counter + 1,
+                                  ctx->stream), "surrogate forward");
     }
     if (flags & FIRE_SYNC) return fire_sync(ctx);
     return FIRE_OK;
@@ -732,13 +817,9 @@ int fire_net_backward(fire_ctx *ctx, fire_net *net, int n, const uint16_t *x,
     cudaStream_t st = ctx->stream;
     uint32_t *err = ctx->counter + 1;
     const int S = net->S, lgS = net->lgS, P = n * S * S;
-    CUDA_TRY(ctx, net_forward(net, n, x, err, st), "surrogate forward");
     CUDA_TRY(ctx, cudaMemsetAsync(net->loss, 0, 8, st), "loss clear");
     CUDA_TRY(ctx, cudaMemsetAsync(net->grad, 0, (size_t)kParams * 4, st), "grad clear");
-    k_head<<<(P + 255) / 256, 256, 0, st>>>(net->h[kL - 1], net->theta + kHead, P,
-                                            target, 1.0f / (float)P, net->prob,
-                                            net->g, net->loss);
-    CUDA_TRY(ctx, cudaGetLastError(), "surrogate head");
+    CUDA_TRY(ctx, net_forward(net, n, x, net->prob, target, err, st), "surrogate forward");
     const int per = 256;
     const int nblk = (P + per - 1) / per;
     k_head_grad<<<nblk, 256, 0, st>>>(net->h[kL - 1], net->theta + kHead, net->g, P,
@@ -770,8 +851,8 @@ int fire_net_backward(fire_ctx *ctx, fire_net *net, int n, const uint16_t *x,
             const uint16_t *wt = net->wt + (size_t)(l - 1) * kWl;
             if (S >= 16) {
                 CUDA_TRY(ctx, launch_conv_tma(1, net->dz[l], wt, nullptr, net->h[l - 1],
-                                              net->dz[l - 1], n, S, lgS, kDil[l], err,
-                                              st), "input gradient");
+                                              net->dz[l - 1], n, S, lgS, kDil[l], nullptr,
+                                              err, st), "input gradient");
             } else {
                 ConvDgrad p{net->dz[l], wt, net->h[l - 1], net->dz[l - 1], P, kC,
                             9 * kC, S, lgS, kDil[l]};
@@ -854,9 +935,14 @@ int fire_net_inputs(fire_ctx *ctx, int S, int H, int W, int n, const float *plan
     if (n == 0) return FIRE_OK;
     int rc = ensure_device(ctx);
     if (rc) return rc;
-    const long long T = (long long)n * S * S;
-    k_inputs<<<(unsigned)((T + 255) / 256), 256, 0, ctx->stream>>>(S, H, W, n, planes,
-                                                                   params, ign, x);
+    const unsigned blocks = (unsigned)(((long long)S * S + 255) / 256);
+    // the grid's second dimension holds 65535 groups of samples
+    for (long long s0 = 0; s0 < n; s0 += 65535ll * kInputSamples) {
+        const int ns = (int)std::min<long long>(n - s0, 65535ll * kInputSamples);
+        k_inputs<<<dim3(blocks, (ns + kInputSamples - 1) / kInputSamples), 256, 0,
+                   ctx->stream>>>(S, H, W, ns, planes, params + s0, ign + s0,
+                                  x + (size_t)s0 * S * S * kCin);
+    }
     CUDA_TRY(ctx, cudaGetLastError(), "inputs");
     if (flags & FIRE_SYNC) return fire_sync(ctx);
     return FIRE_OK;
@@ -948,9 +1034,27 @@ int fire_net_screen(fire_ctx *ctx, int S, int n, const float *prob,
     if (n == 0) return FIRE_OK;
     int rc = ensure_device(ctx);
     if (rc) return rc;
-    k_pred_fitness<<<n, 256, 0, ctx->stream>>>(S * S, prob, target_frac,
-                                               cells_per_coarse, kind, pred);
-    CUDA_TRY(ctx, cudaGetLastError(), "predicted fitness");
+    // eight blocks per candidate where that fills more of the chip and each has
+    // at least four cells a thread
+    if (S * S >= 8192 && n < 8 * ctx->num_sms) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)n * 8);
+        cfg.blockDim = dim3(256);
+        cfg.stream = ctx->stream;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = 8;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        CUDA_TRY(ctx, cudaLaunchKernelEx(&cfg, k_pred_fitness<8>, S * S, prob, target_frac,
+                                         cells_per_coarse, kind, pred),
+                 "predicted fitness");
+    } else {
+        k_pred_fitness<1><<<n, 256, 0, ctx->stream>>>(S * S, prob, target_frac,
+                                                      cells_per_coarse, kind, pred);
+        CUDA_TRY(ctx, cudaGetLastError(), "predicted fitness");
+    }
     if (keep) {
         k_rank_keep<<<(n + 127) / 128, 128, 0, ctx->stream>>>(n, pred, keep, keep_idx);
         CUDA_TRY(ctx, cudaGetLastError(), "rank");
