@@ -172,6 +172,19 @@ __device__ __forceinline__ void tma_4d_pair(uint32_t dst, const CUtensorMap *map
         : "memory");
 }
 
+__device__ __forceinline__ void tma_5d_pair(uint32_t dst, const CUtensorMap *map,
+                                            int c0, int c1, int c2, int c3, int c4,
+                                            uint32_t bar)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.5d.cta_group::2.shared::cluster.global.tile."
+        "mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5, %6}], [%7];" ::"r"(
+            dst),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3),
+        "r"(c4), "r"(bar)
+        : "memory");
+}
+
 __device__ __forceinline__ void tma_2d_pair(uint32_t dst, const CUtensorMap *map,
                                             int c0, int c1, uint32_t bar)
 {
@@ -193,6 +206,15 @@ __device__ __forceinline__ void mma_bf16_pair(uint32_t d_tmem, uint64_t adesc,
             d_tmem),
         "l"(adesc), "l"(bdesc), "r"(idesc), "r"((uint32_t)accumulate)
         : "memory");
+}
+
+// The four K = 16 steps of a 64-wide slab.
+__device__ __forceinline__ void issue4(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
+                                       uint32_t idesc, bool accumulate)
+{
+#pragma unroll
+    for (int kk = 0; kk < 4; ++kk)
+        mma_bf16_pair(d_tmem, adesc + kk * 2, bdesc + kk * 2, idesc, accumulate || kk > 0);
 }
 
 // Arrives on the barrier at this offset in both CTAs once the MMAs issued so
@@ -226,9 +248,13 @@ __device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols
 
 // How the pair convolution streams a layer's activations (conv_shape): strips
 // of `px` pixels x 64 channels, each serving `taps` taps (the three of a row,
-// or one), in `na` shared-memory stages.
+// or one), in `na` shared-memory stages.  comb > 0: a CTA's 128 pixels are a
+// comb of the row, `comb` neighbouring pixels at every multiple of d, so that a
+// tap's shift by d is a shift by one tooth within the same 128 pixels; beyond
+// the first and the last tooth the row ends, and a gap of `comb` zero pixels
+// between the stages stands for both.
 struct StripShape {
-    int taps, px, na;
+    int taps, px, na, comb;
 };
 
 constexpr int kWHalf = 64 * 128;                // 64 weight rows x 64 BF16
@@ -339,10 +365,11 @@ __device__ __forceinline__ void pair_epilogue(const Epi &epi, const float *s_bia
 //    descriptor arithmetic per 64-wide slab it took 500 clocks a slab
 //    whatever the MMA count, against 256 for the slab's MMAs.  Waits and
 //    commits per row of taps, unrolled, leave the tensor core the bound.
-// Measured (one layer, 1909 TFLOP/s measured peak): 90 us for d <= 16 (1718
-// TFLOP/s), 126 us for d = 32 (three strips, one in flight), 135 us for
-// d = 64; one 128-pixel tile per CTA with boxes per tap and streamed weights
-// took 136 us for every d.
+// Measured (one layer): 84.5 us for d <= 16 (1830 TFLOP/s) and, with combs, for
+// d = 32; 110 us for d = 64 (combs, three stages); the input gradients, which
+// also read the layer below's activations, 95 and 114.  One 128-pixel tile per
+// CTA with boxes per tap and streamed weights took 136 us for every d, and 158
+// for the input gradients.
 //
 // Persistent: one pair per two SMs walks pairs of tiles.  In both CTAs one
 // thread issues the strip copies, whose bytes count on the leader's barrier
@@ -352,11 +379,12 @@ __device__ __forceinline__ void pair_epilogue(const Epi &epi, const float *s_bia
 //
 // sign = +1: forward (source pixel p + off(t)); -1: input gradient (p - off(t)).
 // A strip of `px` pixels serves kTaps taps (StripShape); `na` strip stages.
-template <int kTaps, int kMode>
+// kComb: kTaps is 3 and the tiles are combs.
+template <int kTaps, int kMode, bool kComb>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
     k_conv_pair(const __grid_constant__ CUtensorMap act,
-                const __grid_constant__ CUtensorMap wts, Epi epi, int px, int na, int S,
-                int lgS, int d, int sign, int npairs, uint32_t *err)
+                const __grid_constant__ CUtensorMap wts, Epi epi, int px, int na, int comb,
+                int S, int lgS, int d, int sign, int npairs, uint32_t *err)
 {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     const uint32_t raw = tc::smem_addr(smem_raw);
@@ -368,6 +396,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int rank = (int)cluster_rank();
     const int pair0 = blockIdx.x >> 1, pstep = gridDim.x >> 1;
+    constexpr int kGroups = 9 / kTaps;
+    const uint32_t strip = (uint32_t)px * 128;       // from one stage to the next
+    const uint32_t copied = kComb ? 128 * 128 : strip;
+    if (kComb) {
+        // the zero gaps: before each stage's 128 pixels, and behind the last
+        uint4 *const gap = reinterpret_cast<uint4 *>(smem_raw + (abase - raw));
+        const int n16 = comb * 8;
+        for (int i = tid; i < (na + 1) * n16; i += kPairThreads)
+            gap[(i / n16) * (strip >> 4) + i % n16] = make_uint4(0u, 0u, 0u, 0u);
+        tc::fence_proxy_async();
+    }
     if (kMode != kDgrad && tid < 128) sh.bias[tid] = epi.bias[tid];
     if (kMode == kFwdHead && tid <= 128) sh.head[tid] = epi.head.wh[tid];
     if (warp == kEpiWarps) tmem_alloc_pair(&sh.tmem_slot, 256);
@@ -391,8 +430,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
     cluster_sync();   // the barriers of both CTAs are set up
     tc::fence_after_sync();
     const uint32_t tmem = sh.tmem_slot;
-    const uint32_t strip = (uint32_t)px * 128;
-    constexpr int kGroups = 9 / kTaps;
 
     if (warp == kEpiWarps) {
         // strip loader: strip g of the pair's sequence uses stage g mod na
@@ -412,9 +449,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
                     ok = all_ok(ok && !*(volatile int *)&sh.fail);
                     if (!ok) break;
                     if (leader) {
-                        if (rank == 0) expect_tx(&sh.afull[st], 2 * strip);
-                        tma_4d_pair(abase + st * strip, &act, half * 64, x0 + dx, y0 + dy,
-                                    b, leader_addr(&sh.afull[st]));
+                        if (rank == 0) expect_tx(&sh.afull[st], 2 * copied);
+                        if (kComb)
+                            tma_5d_pair(abase + st * strip + comb * 128, &act, half * 64,
+                                        (x0 >> 7) * comb, 0, y0 + dy, b,
+                                        leader_addr(&sh.afull[st]));
+                        else
+                            tma_4d_pair(abase + st * strip, &act, half * 64, x0 + dx,
+                                        y0 + dy, b, leader_addr(&sh.afull[st]));
                     }
                     __syncwarp();
                     if (++st == na) st = 0, ph ^= 1;
@@ -451,8 +493,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
             const uint32_t strip16 = strip >> 4;
             // rows of a strip: a tap's shift (a multiple of 128 bytes; the
             // 128-byte swizzle goes by address, so any row may come first)
-            const uint32_t row0 = sign > 0 ? 0 : (kTaps - 1) * (uint32_t)d * 8;
-            const int rowstep = sign * d * 8;
+            const int shift = kComb ? comb : d;
+            const uint32_t row0 = sign > 0 ? 0 : (kTaps - 1) * (uint32_t)shift * 8;
+            const int rowstep = sign * shift * 8;
             const bool leader = elect_one();
             int it = 0, ast = 0, ag = 0;
             uint32_t aph = 0;
@@ -469,25 +512,33 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
                     if (it == 0)
                         for (int s = 2 * kTaps * q; ok && s < 2 * kTaps * (q + 1); ++s)
                             ok = all_ok(tc::mbar_wait_bounded(&sh.wfull[s], 0));
-                    ok = ok && all_ok(tc::mbar_wait_bounded(&sh.afull[st0], aph) &&
-                                      tc::mbar_wait_bounded(&sh.afull[st1], ph1));
+                    ok = ok && all_ok(tc::mbar_wait_bounded(&sh.afull[st0], aph));
                     if (!ok) break;
                     tc::fence_after_sync();
                     const uint64_t a0 = adesc + st0 * strip16 + row0;
                     const uint64_t a1 = adesc + st1 * strip16 + row0;
                     const uint64_t w0 = wdesc + q * (2 * kTaps * (kWHalf >> 4));
+                    // the first tap's first half starts without the second strip,
+                    // and the first strip is released before the last half: what
+                    // three strips need to keep one in flight (d = 64 at S = 256:
+                    // 110 us against 128)
+                    if (kTaps == 3) {
+                        if (leader) issue4(td, a0, w0, idesc, q > 0);
+                        __syncwarp();
+                    }
+                    ok = all_ok(tc::mbar_wait_bounded(&sh.afull[st1], ph1));
+                    if (!ok) break;
+                    tc::fence_after_sync();
                     if (leader) {
 #pragma unroll
-                        for (int j = 0; j < kTaps; ++j)
-#pragma unroll
-                            for (int h = 0; h < 2; ++h)
-#pragma unroll
-                                for (int kk = 0; kk < 4; ++kk)
-                                    mma_bf16_pair(
-                                        td, (h ? a1 : a0) + j * rowstep + kk * 2,
-                                        w0 + (2 * j + h) * (kWHalf >> 4) + kk * 2, idesc,
-                                        q > 0 || j > 0 || h > 0 || kk > 0);
-                        commit_pair(&sh.aempty[st0]);
+                        for (int j = 0; j < kTaps; ++j) {
+                            if (j > 0 || kTaps == 1)
+                                issue4(td, a0 + j * rowstep, w0 + 2 * j * (kWHalf >> 4),
+                                       idesc, q > 0 || j > 0);
+                            if (j == kTaps - 1) commit_pair(&sh.aempty[st0]);
+                            issue4(td, a1 + j * rowstep,
+                                   w0 + (2 * j + 1) * (kWHalf >> 4), idesc, true);
+                        }
                         commit_pair(&sh.aempty[st1]);
                         if (q == kGroups - 1) commit_pair(&sh.tfull[acc]);
                     }
@@ -509,7 +560,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
         int it = 0;
         for (int pr = pair0; pr < npairs; pr += pstep, ++it) {
             const int acc = it & 1;
-            const size_t p = (size_t)(2 * pr + rank) * 128 + warp * 32 + lane;
+            const int tile = 2 * pr + rank, m = warp * 32 + lane;
+            size_t p = (size_t)tile * 128 + m;
+            if (kComb) {
+                // tile of the row: its tooth; pixel m: tooth m / comb, then m mod comb
+                const int r = tile >> (lgS - 7), c = tile & ((S >> 7) - 1);
+                const int tooth = m / comb;
+                p = ((size_t)r << lgS) + tooth * d + c * comb + (m - tooth * comb);
+            }
             uint32_t mask[64];
             if (kMode == kDgrad) {
 #pragma unroll
@@ -999,14 +1057,43 @@ bool map_act(CUtensorMap *m, const uint16_t *ptr, int n, int S, int pix = 128)
 }
 
 // Strips of the pair convolution.  Three taps share a strip when a CTA's 128
-// pixels lie in one row (S >= 128) and three strips fit in shared memory (two
-// serve a row of taps, one is filled meanwhile): dilations up to 32.
+// pixels lie in one row (S >= 128) and its stages fit: two strips serve a row
+// of taps, and with four the next row's are on their way (dilations up to 16:
+// 84.5 us a layer at 8 x 256 x 256; three strips of 192 pixels, d = 32, took 126
+// and a box per tap, d = 64, 135).  Combs stream 128 pixels per strip whatever d
+// and fit three or four from d = 32 on (85.8 and 110 us); their teeth are 128 d
+// / S pixels wide and whole 1 KB groups.
 StripShape conv_shape(int S, int d)
 {
-    StripShape sp{3, 128 + (2 * d + 7) / 8 * 8, 0};
-    if (S < 128 || 3 * sp.px * 128 > kStripRoom) sp = StripShape{1, 128, 0};
-    sp.na = std::min(kMaxA, kStripRoom / (sp.px * 128));
-    return sp;
+    StripShape sp{3, 128 + (2 * d + 7) / 8 * 8, 0, 0};
+    if (S >= 128) {
+        sp.na = std::min(4, kStripRoom / (sp.px * 128));
+        const int tooth = 128 * d / S;
+        if (sp.na < 4 && d < S && tooth >= 8) {
+            const int na = std::min(4, (kStripRoom - tooth * 128) / ((128 + tooth) * 128));
+            if (na >= 3 && na >= sp.na) return StripShape{3, 128 + tooth, na, tooth};
+        }
+        if (sp.na >= 3) return sp;
+    }
+    return StripShape{1, 128, kMaxA, 0};
+}
+
+// NHWC activations of 128 channels with x split into (x mod d, x / d): box 64
+// channels x w pixels x all S / d multiples of one row.
+bool map_comb(CUtensorMap *m, const uint16_t *ptr, int n, int S, int d, int w)
+{
+    auto fn = encoder();
+    if (!fn) return false;
+    const cuuint64_t dims[5] = {128, (cuuint64_t)d, (cuuint64_t)(S / d), (cuuint64_t)S,
+                                (cuuint64_t)n};
+    const cuuint64_t strides[4] = {256, (cuuint64_t)d * 256, (cuuint64_t)S * 256,
+                                   (cuuint64_t)S * S * 256};
+    const cuuint32_t box[5] = {64, (cuuint32_t)w, (cuuint32_t)(S / d), 1, 1};
+    const cuuint32_t es[5] = {1, 1, 1, 1, 1};
+    return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<uint16_t *>(ptr), dims,
+              strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+              CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 // NHWC tensor of 128 (box 64, 128-byte swizzle) or 16 channels (32-byte
@@ -1095,17 +1182,24 @@ cudaError_t launch_conv_tma(int mode, const uint16_t *in, const uint16_t *w,
         return cudaErrorInvalidValue;
     const StripShape sp = conv_shape(S, d);
     CUtensorMap ma, mw;
-    if (!map_act(&ma, in, n, S, sp.px) || !map_wts(&mw, w)) return cudaErrorInvalidValue;
+    if (!(sp.comb ? map_comb(&ma, in, n, S, d, sp.comb) : map_act(&ma, in, n, S, sp.px)) ||
+        !map_wts(&mw, w))
+        return cudaErrorInvalidValue;
     Epi e{bias, hprev, out, head ? *head : HeadArgs{}};
     int dev = 0, nsm = 0;
     cudaError_t attr = cudaGetDevice(&dev);
     if (attr == cudaSuccess)
         attr = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    const bool three = sp.taps == 3;
-    const auto kern =
-        mode != 0 ? (three ? k_conv_pair<3, kDgrad> : k_conv_pair<1, kDgrad>)
-        : head    ? (three ? k_conv_pair<3, kFwdHead> : k_conv_pair<1, kFwdHead>)
-                  : (three ? k_conv_pair<3, kFwd> : k_conv_pair<1, kFwd>);
+    using Kernel = decltype(&k_conv_pair<3, kFwd, true>);
+    static const Kernel kerns[3][3] = {   // mode x (boxes, strips, combs)
+        {k_conv_pair<1, kFwd, false>, k_conv_pair<3, kFwd, false>,
+         k_conv_pair<3, kFwd, true>},
+        {k_conv_pair<1, kDgrad, false>, k_conv_pair<3, kDgrad, false>,
+         k_conv_pair<3, kDgrad, true>},
+        {k_conv_pair<1, kFwdHead, false>, k_conv_pair<3, kFwdHead, false>,
+         k_conv_pair<3, kFwdHead, true>}};
+    const Kernel kern = kerns[mode != 0 ? kDgrad : head ? kFwdHead : kFwd]
+                             [sp.comb ? 2 : sp.taps == 3 ? 1 : 0];
     if (attr == cudaSuccess)
         attr = cudaFuncSetAttribute(
             kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kPairSmem);
@@ -1113,7 +1207,7 @@ cudaError_t launch_conv_tma(int mode, const uint16_t *in, const uint16_t *w,
     // S >= 16: whole pairs of 128-pixel tiles
     const int npairs = (int)((long long)n * S * S / 256);
     kern<<<2 * std::min(npairs, nsm / 2), kPairThreads, kPairSmem, st>>>(
-        ma, mw, e, sp.px, sp.na, S, lgS, d, mode == 0 ? 1 : -1, npairs, err);
+        ma, mw, e, sp.px, sp.na, sp.comb, S, lgS, d, mode == 0 ? 1 : -1, npairs, err);
     return cudaGetLastError();
 }
 
