@@ -433,6 +433,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
 
     if (warp == kEpiWarps) {
         // strip loader: strip g of the pair's sequence uses stage g mod na
+        pdl_wait();
         const bool leader = elect_one();
         int g = 0, st = 0;
         uint32_t ph = 1;   // parity of the stage's last release
@@ -469,7 +470,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
         }
         __syncwarp();
     } else if (warp == kEpiWarps + 1) {
-        // this CTA's half of the weights: rows 64 rank .. 64 rank + 63
+        // this CTA's half of the weights: rows 64 rank .. 64 rank + 63 (no
+        // kernel that can still be running writes them)
         const bool leader = elect_one();
         for (int s = 0; s < kSlabs; ++s) {
             if (leader) {
@@ -557,6 +559,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
         }
     } else {
         // epilogue: pair number `it` is read from buffer it & 1
+        pdl_wait();
         int it = 0;
         for (int pr = pair0; pr < npairs; pr += pstep, ++it) {
             const int acc = it & 1;
@@ -710,6 +713,7 @@ __global__ void __launch_bounds__(kWgThreads, 1)
     __syncthreads();
     tc::fence_after_sync();
     const uint32_t tmem = sh.tmem_slot;
+    pdl_wait();
 
     if (warp == 4) {
         const bool leader = elect_one();
@@ -894,7 +898,6 @@ __global__ void __launch_bounds__(kC1Threads, 1)
                                                  kC1Stages * kStage + 9 * kC1Tile);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    if (tid < 128) sh.bias[tid] = epi.bias[tid];
     if (warp == 8) {
         tc::tmem_alloc(&sh.tmem_slot, 512);
         tc::tmem_relinquish();
@@ -913,6 +916,10 @@ __global__ void __launch_bounds__(kC1Threads, 1)
         sh.fail = sh.issued = sh.used = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    // the optimiser's step, which writes weights and biases, may be the kernel
+    // before this one
+    pdl_wait();
+    if (tid < 128) sh.bias[tid] = epi.bias[tid];
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
@@ -1206,9 +1213,9 @@ cudaError_t launch_conv_tma(int mode, const uint16_t *in, const uint16_t *w,
     if (attr != cudaSuccess) return attr;
     // S >= 16: whole pairs of 128-pixel tiles
     const int npairs = (int)((long long)n * S * S / 256);
-    kern<<<2 * std::min(npairs, nsm / 2), kPairThreads, kPairSmem, st>>>(
-        ma, mw, e, sp.px, sp.na, sp.comb, S, lgS, d, mode == 0 ? 1 : -1, npairs, err);
-    return cudaGetLastError();
+    return launch_pdl(kern, dim3(2 * std::min(npairs, nsm / 2)), kPairThreads, kPairSmem, st,
+                      ma, mw, e, sp.px, sp.na, sp.comb, S, lgS, d, mode == 0 ? 1 : -1, npairs,
+                      err);
 }
 
 // Weight gradient, added into dw[128][9 cin] (FP32, cleared by the caller), and
@@ -1243,9 +1250,8 @@ cudaError_t launch_wgrad_tma(const uint16_t *dz, const uint16_t *in, int cin, fl
     const int total = (int)((long long)n * S * S / sp.L);
     const int rows = cin == 128 ? 3 : 1;   // rows of taps, one per CTA
     const int per = (total + nsm / rows - 1) / (nsm / rows);
-    kern<<<dim3((total + per - 1) / per, rows), kWgThreads, smem, st>>>(
-        mz, mi, dw, db, S, lgS, d, sp, total, per, err);
-    return cudaGetLastError();
+    return launch_pdl(kern, dim3((total + per - 1) / per, rows), kWgThreads, smem, st, mz, mi,
+                      dw, db, S, lgS, d, sp, total, per, err);
 }
 
 // First layer forward: out = ReLU(conv3x3(x, W1) + b1) for x [n][S][S][16]
@@ -1273,8 +1279,8 @@ cudaError_t launch_conv1_tma(const uint16_t *x, const uint16_t *w, const float *
         attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (attr != cudaSuccess) return attr;
     const int ntiles = (int)((long long)n * S * S / 128);
-    kern<<<std::min(ntiles, nsm), kC1Threads, smem, st>>>(ma, mw, e, S, lgS, ntiles, err);
-    return cudaGetLastError();
+    return launch_pdl(kern, dim3(std::min(ntiles, nsm)), kC1Threads, smem, st, ma, mw, e, S,
+                      lgS, ntiles, err);
 }
 
 }  // namespace fire

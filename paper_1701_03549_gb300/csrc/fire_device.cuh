@@ -18,6 +18,13 @@
 
 namespace fire {
 
+// Wait for the grids this launch depends on (launch_pdl in fire_internal.h);
+// then let the next one begin as CTAs leave.
+__device__ __forceinline__ void pdl_wait()
+{
+    asm volatile("griddepcontrol.wait;\n\tgriddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // ---------------------------------------------------------------------------
 // Philox4x32-10 (Salmon, Moraes, Dror, Shaw, SC'11).  Round:
 //   (hi0, lo0) = M0 * x0, (hi1, lo1) = M1 * x2,

@@ -271,6 +271,28 @@ int noalloc_take_error(int device, bool *set);
 // grown, so a state that fits in shared memory goes there).
 int plan_launch(fire_ctx *ctx, int ntiles, long long n, LaunchPlan *p,
                 bool burn = false, bool fixed_scratch = false);
+// Launch that may begin while the kernel before it on the stream drains
+// (programmatic stream serialisation).  The kernel calls pdl_wait() before it
+// touches anything an earlier kernel wrote or reads; what comes before that
+// (barriers, tensor memory, weights, which no kernel of a pass writes) overlaps
+// the predecessor's last CTAs.
+template <class Kernel, class... Args>
+cudaError_t launch_pdl(Kernel kern, dim3 grid, int threads, size_t smem, cudaStream_t st,
+                       Args... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
 // The network's head on the top layer's activations: probabilities, and with
 // target the per-pixel gradient g and the loss terms (summed by k_loss_sum).
 struct HeadArgs {

@@ -239,6 +239,7 @@ __global__ void __launch_bounds__(256)
     k_loss_sum(const float2 *__restrict__ term, int P, int nw, float inv_count,
                double *__restrict__ loss)
 {
+    pdl_wait();
     const int w = blockIdx.x * blockDim.x + threadIdx.x;
     float l0 = 0.0f, l1 = 0.0f;
     if (w < nw)
@@ -268,6 +269,7 @@ __global__ void __launch_bounds__(256)
                 uint16_t *__restrict__ dz, float *__restrict__ dwh)
 {
     __shared__ float red[16][kC + 2];
+    pdl_wait();
     const int cg = threadIdx.x & 15, pl = threadIdx.x >> 4;
     const int p0 = blockIdx.x * per, p1 = min(P, p0 + per);
     float w[8];
@@ -652,8 +654,9 @@ cudaError_t net_forward(fire_net *net, int n, const uint16_t *x, float *prob,
                                             inv_count, prob, net->g, net->loss);
     } else if (target) {
         const int nw = head_blocks * 8;
-        k_loss_sum<<<(nw + 255) / 256, 256, 0, st>>>(
-            reinterpret_cast<const float2 *>(net->term), M, nw, inv_count, net->loss);
+        return launch_pdl(k_loss_sum, dim3((nw + 255) / 256), 256, 0, st,
+                          reinterpret_cast<const float2 *>(net->term), M, nw, inv_count,
+                          net->loss);
     }
     return cudaGetLastError();
 }
@@ -822,9 +825,11 @@ int fire_net_backward(fire_ctx *ctx, fire_net *net, int n, const uint16_t *x,
     CUDA_TRY(ctx, net_forward(net, n, x, net->prob, target, err, st), "surrogate forward");
     const int per = 256;
     const int nblk = (P + per - 1) / per;
-    k_head_grad<<<nblk, 256, 0, st>>>(net->h[kL - 1], net->theta + kHead, net->g, P,
-                                     per, net->dz[kL - 1], net->grad + kHead);
-    CUDA_TRY(ctx, cudaGetLastError(), "head gradient");
+    CUDA_TRY(ctx, launch_pdl(k_head_grad, dim3(nblk), 256, 0, st,
+                             (const uint16_t *)net->h[kL - 1],
+                             (const float *)(net->theta + kHead), (const float *)net->g, P,
+                             per, net->dz[kL - 1], net->grad + kHead),
+             "head gradient");
     const int kslabs = P / 64;
     for (int l = kL - 1; l >= 0; --l) {
         cudaError_t e;
