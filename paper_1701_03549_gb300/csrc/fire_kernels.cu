@@ -845,7 +845,22 @@ __global__ void __launch_bounds__(kSimMaxThreads, 2) k_simulate(SimLaunch a)
         }
         if (a.burn_step) {
             int32_t *bs = a.burn_step + (long long)sim * HW;
-            for (long long i = threadIdx.x; i < HW; i += blockDim.x)
+            // eight cells at a time where both arrays allow 16-byte accesses
+            const long long n8 = ((uintptr_t)bs & 15) == 0 ? HW / 8 : 0;
+            for (long long i = threadIdx.x; i < n8; i += blockDim.x) {
+                const uint4 f = __ldg(reinterpret_cast<const uint4 *>(m.cfl) + i);
+                const uint32_t w4[4] = {f.x, f.y, f.z, f.w};
+                int32_t v[8];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    v[2 * j] = (w4[j] & kFlagBurnable) ? -1 : -2;
+                    v[2 * j + 1] = ((w4[j] >> 16) & kFlagBurnable) ? -1 : -2;
+                }
+                int4 *o = reinterpret_cast<int4 *>(bs) + 2 * i;
+                o[0] = make_int4(v[0], v[1], v[2], v[3]);
+                o[1] = make_int4(v[4], v[5], v[6], v[7]);
+            }
+            for (long long i = 8 * n8 + threadIdx.x; i < HW; i += blockDim.x)
                 bs[i] = (m.cfl[i] & kFlagBurnable) ? -1 : -2;
         }
         if (kSmemState) {
