@@ -221,6 +221,10 @@ int fire_create(fire_ctx **out, int device, void *cuda_stream)
         ctx->own_stream = true;
     }
     e = cudaMalloc(&ctx->counter, 256);
+    if (e == cudaSuccess) {
+        e = cudaMallocHost(&ctx->host_error, 64);
+        if (e != cudaSuccess) cudaFree(ctx->counter);
+    }
     if (e != cudaSuccess) {
         if (ctx->own_stream) cudaStreamDestroy(ctx->stream);
         delete ctx;
@@ -241,6 +245,7 @@ void fire_destroy(fire_ctx *ctx)
     if (ctx->order) cudaFree(ctx->order);
     if (ctx->lpt) cudaFree(ctx->lpt);
     if (ctx->counter) cudaFree(ctx->counter);
+    if (ctx->host_error) cudaFreeHost(ctx->host_error);
     if (ctx->staging) cudaFree(ctx->staging);
     if (ctx->gstate) cudaFree(ctx->gstate);
     if (ctx->burn_aux) cudaFree(ctx->burn_aux);
@@ -260,11 +265,13 @@ int fire_sync(fire_ctx *ctx)
     if (!ctx) return FIRE_EINVAL;
     int rc = ensure_device(ctx);
     if (rc) return rc;
-    CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream), "cudaStreamSynchronize");
-    uint32_t errw = 0;
-    CUDA_TRY(ctx, cudaMemcpy(&errw, ctx->counter + 1, 4, cudaMemcpyDeviceToHost),
+    // the error word comes back with the work it belongs to: one wait, where a
+    // blocking copy after the synchronisation was a second round trip
+    CUDA_TRY(ctx, cudaMemcpyAsync(ctx->host_error, ctx->counter + 1, 4,
+                                  cudaMemcpyDeviceToHost, ctx->stream),
              "read error word");
-    if (errw) {
+    CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream), "cudaStreamSynchronize");
+    if (*ctx->host_error) {
         cudaMemset(ctx->counter + 1, 0, 4);
         return set_err(ctx, FIRE_ETIMEOUT, "a bounded device wait ran out");
     }
@@ -550,7 +557,7 @@ int launch_batch(fire_ctx *ctx, const fire_map *m, int n,
     a.max_steps = max_steps;
     a.qcap = plan.qcap;
     a.cell_uniform = (flags & FIRE_CELL_UNIFORM) ? 1 : 0;
-    cudaError_t e = cudaMemsetAsync(ctx->counter, 0, 4, ctx->stream);
+    cudaError_t e = reset_counter(ctx->counter, grid, n, ctx->stream);
     if (e == cudaSuccess)
         e = launch_simulate(a, smem_state, plan.nwarps, (int)grid, plan.L.total,
                             ctx->stream);

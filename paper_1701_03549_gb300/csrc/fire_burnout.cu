@@ -168,7 +168,7 @@ extern "C" int fire_simulate_burnout(fire_ctx *ctx, const fire_map *m, int n,
     a.max_steps = max_steps;
     a.qcap = plan.qcap;
     a.cell_uniform = 0;
-    cudaError_t e = cudaMemsetAsync(ctx->counter, 0, 4, ctx->stream);
+    cudaError_t e = reset_counter(ctx->counter, plan.grid, n, ctx->stream);
     if (e == cudaSuccess)
         e = launch_simulate_burn(a, plan.nwarps, plan.grid, plan.L.total, ctx->stream);
     if (e == cudaSuccess && !dev) {

@@ -57,7 +57,8 @@ struct SimLaunch {
     uint32_t *burnt_bits;      // nullable; single-map launches only: the final
                                // burnt words (tile-major, blocked cells
                                // cleared), ntiles * 32 words per simulation
-    uint32_t *work_counter;    // zeroed before launch
+    uint32_t *work_counter;    // zeroed before a launch of fewer blocks than
+                               // simulations (reset_counter)
     uint32_t *gstate;          // global-state variant: block_words words per block
     size_t block_words;        // 0: 2 * ntiles_max * 32 (the (X, Y) pairs)
     const uint8_t *burn_time;  // burn-time variant: steps each cell burns
@@ -88,6 +89,7 @@ struct SimShared {
     FxParams fx;
     int use_fx;           // the map and the parameters fit the fixed-point screen
     uint32_t key0, key1;
+    uint32_t first;       // the block's first simulation, then ~0
     int sim;
     int skip;
     int timeout;
@@ -149,6 +151,12 @@ cudaError_t launch_simulate(const SimLaunch &a, bool smem_state, int nwarps,
 // The burn-time variant (global-memory state only).
 cudaError_t launch_simulate_burn(const SimLaunch &a, int nwarps, int grid,
                                  size_t smem_bytes, cudaStream_t st);
+// Clears the work counter for a launch of `grid` blocks over n simulations, if
+// that launch reads it: with a block per simulation it does not.
+inline cudaError_t reset_counter(uint32_t *counter, long long grid, int n, cudaStream_t st)
+{
+    return grid < n ? cudaMemsetAsync(counter, 0, 4, st) : cudaSuccess;
+}
 // Tile-major bit plane of the cells whose burn time is 2 or more, and a flag
 // set when there is any (zeroed by the launcher).
 cudaError_t launch_long_burn(const MapDev &m, const uint8_t *burn_time,
@@ -220,6 +228,7 @@ struct fire_ctx {
     std::string err;
     // device scratch
     uint32_t *counter = nullptr;     // work counter + error word
+    uint32_t *host_error = nullptr;  // pinned copy of the error word (fire_sync)
     void *staging = nullptr;         // inputs / outputs of host-pointer calls
     size_t staging_bytes = 0;
     uint32_t *gstate = nullptr;      // global-state simulation buffers

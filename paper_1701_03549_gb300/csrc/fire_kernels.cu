@@ -3,7 +3,8 @@
 // burnt-map comparison of Eq. 2 fused into it, fitness, and debug exports.
 //
 // Simulation kernel design (one thread block per simulation at a time,
-// persistent blocks pulling simulations from a global counter):
+// persistent blocks, the first simulation of each by its index and the next
+// ones from a global counter):
 //  * State: two bit planes X, Y (one bit per cell each) in 32 x 32-cell tiles,
 //    tile-major, in shared memory when they fit (else in a per-block global
 //    buffer).  A cell's 2-bit code is 00 burnable and unburnt, 11 burnt or
@@ -751,12 +752,19 @@ __global__ void __launch_bounds__(kSimMaxThreads, 2) k_simulate(SimLaunch a)
         mbar_init(&sh.mbar, 1);
         fence_proxy_async_smem();
     }
+    if (threadIdx.x == 0) sh.first = blockIdx.x;
     uint32_t phase = 0;
     __syncthreads();
 
     for (;;) {
         if (threadIdx.x == 0) {
-            const uint32_t w = atomicAdd(a.work_counter, 1u);
+            // a block's first simulation is its own index; the counter hands out
+            // the ones after the grid's
+            uint32_t w = sh.first;
+            if (w == 0xffffffffu)
+                w = gridDim.x < (uint32_t)a.n ? gridDim.x + atomicAdd(a.work_counter, 1u)
+                                              : (uint32_t)a.n;
+            sh.first = 0xffffffffu;
             sh.sim = w < (uint32_t)a.n ? (a.order ? (int)a.order[w] : (int)w)
                                        : a.n;
         }

@@ -198,7 +198,8 @@ int fire_simulate_multi(fire_ctx *ctx, int nmaps, const fire_map *const *maps,
     auto issue = [&]() -> int {
         CUDA_TRY(ctx, launch_order(n, dmap, nmaps, drank, dcounts, dorder, ctx->stream),
                  "order kernels");
-        CUDA_TRY(ctx, cudaMemsetAsync(ctx->counter, 0, 4, ctx->stream), "counter reset");
+        CUDA_TRY(ctx, reset_counter(ctx->counter, plan.grid, n, ctx->stream),
+                 "counter reset");
         CUDA_TRY(ctx, launch_simulate(a, plan.smem_state, plan.nwarps, plan.grid,
                                       plan.L.total, ctx->stream),
                  "simulate launch");
