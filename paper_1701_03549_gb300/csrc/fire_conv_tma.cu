@@ -628,12 +628,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
 // with 16 all three rows (3 x N = 48); a column of ones beside them gives the
 // bias gradient in the same pass, shared out over the rows' CTAs.
 //
-// What bounds it (128 channels, 8 x 256 x 256, 154.6 GFLOP): shared memory,
-// which a 128 x 192 x 16 MMA reads at 107 bytes a clock (128 x 128 x 16: 128)
-// while the copies write 45.  98.5 us with the bias (d = 64: 103); one tap per
-// CTA with a box per operand loaded 32 KB per 64 pixels and tap: 119 us, and
-// another 27 us for a bias pass over dz.  16 channels: 31 us (bound by reading
-// dz, 134 MB) against 204 on register-staged tiles.
+// What bounds it (128 channels, 8 x 256 x 256, 154.6 GFLOP): the copies, 67 KB
+// per 128 pixels for 1536 clocks of MMAs (halving the MMAs saves a fifth), then
+// shared memory, which a 128 x 192 x 16 MMA reads at 107 bytes a clock.  90 us
+// with the bias (5 of them); one tap per CTA with a box per operand loaded 32 KB
+// per 64 pixels and tap: 119 us, and another 27 us for a bias pass over dz.  16
+// channels: 31 us (bound by reading dz, 134 MB) against 204 on register-staged
+// tiles.
 struct WgradShape {
     int L, lgw;        // pixels of a slab, log2 pixels of its rows
     int pitch;         // pixels from one row of a strip to the next
@@ -687,8 +688,9 @@ __global__ void __launch_bounds__(kWgThreads, 1)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     constexpr uint32_t kDz = kSteps * 16 * 256;     // bytes of a dz slab
     const uint32_t stage = kDz + kB * (uint32_t)sp.strip;
-    const int dyi = Cin == 128 ? (int)blockIdx.y : 0;
-    const int s0 = blockIdx.x * slabs_per;
+    // the CTAs of one pixel range are neighbours: their dz requests meet on the way
+    const int dyi = Cin == 128 ? (int)blockIdx.x : 0;
+    const int s0 = blockIdx.y * slabs_per;
     const int ns = min(slabs_total - s0, slabs_per);
     // slabs whose bias this CTA sums: all, or those of its residue mod 3
     const int nbias = Cin == 128 ? (s0 + ns + 2 - dyi) / 3 - (s0 + 2 - dyi) / 3 : ns;
@@ -772,16 +774,18 @@ __global__ void __launch_bounds__(kWgThreads, 1)
             const bool bias = Cin != 128 || (s0 + s) % 3 == dyi;
             if (leader) {
 #pragma unroll
-                for (int j = 0; j < kSteps; ++j) {
+                for (int j = 0; j < kSteps; ++j)
 #pragma unroll
                     for (int i = 0; i < kB; ++i)
                         tc::mma_bf16(tmem + i * kN, ad + off + j * 128,
                                      bd + off + i * strip16 + row16[j], idesc,
                                      s > 0 || j > 0);
-                    if (bias)
+                // together: between the others each cost 110 clocks
+                if (bias)
+#pragma unroll
+                    for (int j = 0; j < kSteps; ++j)
                         tc::mma_bf16(tmem + kBiasCol, ad + off + j * 128, od, idesc1,
                                      nb > 0 || j > 0);
-                }
                 tc::mma_commit(&sh.empty[st]);
             }
             __syncwarp();
@@ -1250,7 +1254,7 @@ cudaError_t launch_wgrad_tma(const uint16_t *dz, const uint16_t *in, int cin, fl
     const int total = (int)((long long)n * S * S / sp.L);
     const int rows = cin == 128 ? 3 : 1;   // rows of taps, one per CTA
     const int per = (total + nsm / rows - 1) / (nsm / rows);
-    return launch_pdl(kern, dim3((total + per - 1) / per, rows), kWgThreads, smem, st, mz, mi,
+    return launch_pdl(kern, dim3(rows, (total + per - 1) / per), kWgThreads, smem, st, mz, mi,
                       dw, db, S, lgS, d, sp, total, per, err);
 }
 
