@@ -248,13 +248,19 @@ __device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols
 
 // How the pair convolution streams a layer's activations (conv_shape): strips
 // of `px` pixels x 64 channels, each serving `taps` taps (the three of a row,
-// or one), in `na` shared-memory stages.  comb > 0: a CTA's 128 pixels are a
-// comb of the row, `comb` neighbouring pixels at every multiple of d, so that a
-// tap's shift by d is a shift by one tooth within the same 128 pixels; beyond
-// the first and the last tooth the row ends, and a gap of `comb` zero pixels
-// between the stages stands for both.
+// or one), in `na` shared-memory stages.
+//
+// step > 0: the tile's 128 pixels are laid out so that a tap's shift by d pixels
+// is a shift by `step` pixels of the tile itself, and what it shifts in from
+// beyond is the zero padding: `gap` zero pixels between the stages.  Pixel m of
+// the tile is pixel (m / fold) * outer + (m mod fold) * inner of the image.
+//   Row combs (d >= S / 16): `fold` = 128 d / S neighbouring pixels at every
+//     multiple of d of one row; a shift is one tooth.
+//   Columns (S < 128): 128 / S whole rows, column by column; a shift is d
+//     columns.
 struct StripShape {
-    int taps, px, na, comb;
+    int taps, px, na;
+    int step, gap, fold, outer, inner, cols;   // cols: columns, else comb
 };
 
 constexpr int kWHalf = 64 * 128;                // 64 weight rows x 64 BF16
@@ -378,13 +384,13 @@ __device__ __forceinline__ void pair_epilogue(const Epi &epi, const float *s_bia
 // a tile's epilogue runs under the next tile's MMAs.
 //
 // sign = +1: forward (source pixel p + off(t)); -1: input gradient (p - off(t)).
-// A strip of `px` pixels serves kTaps taps (StripShape); `na` strip stages.
-// kComb: kTaps is 3 and the tiles are combs.
+// A strip serves kTaps taps (StripShape).  kComb: kTaps is 3 and the tiles are
+// combs or columns.
 template <int kTaps, int kMode, bool kComb>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
     k_conv_pair(const __grid_constant__ CUtensorMap act,
-                const __grid_constant__ CUtensorMap wts, Epi epi, int px, int na, int comb,
-                int S, int lgS, int d, int sign, int npairs, uint32_t *err)
+                const __grid_constant__ CUtensorMap wts, Epi epi, StripShape sp, int S,
+                int lgS, int d, int sign, int npairs, uint32_t *err)
 {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     const uint32_t raw = tc::smem_addr(smem_raw);
@@ -397,12 +403,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
     const int rank = (int)cluster_rank();
     const int pair0 = blockIdx.x >> 1, pstep = gridDim.x >> 1;
     constexpr int kGroups = 9 / kTaps;
-    const uint32_t strip = (uint32_t)px * 128;       // from one stage to the next
+    const int na = sp.na;
+    const uint32_t strip = (uint32_t)sp.px * 128;    // from one stage to the next
     const uint32_t copied = kComb ? 128 * 128 : strip;
     if (kComb) {
         // the zero gaps: before each stage's 128 pixels, and behind the last
         uint4 *const gap = reinterpret_cast<uint4 *>(smem_raw + (abase - raw));
-        const int n16 = comb * 8;
+        const int n16 = sp.gap * 8;
         for (int i = tid; i < (na + 1) * n16; i += kPairThreads)
             gap[(i / n16) * (strip >> 4) + i % n16] = make_uint4(0u, 0u, 0u, 0u);
         tc::fence_proxy_async();
@@ -452,8 +459,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
                     if (leader) {
                         if (rank == 0) expect_tx(&sh.afull[st], 2 * copied);
                         if (kComb)
-                            tma_5d_pair(abase + st * strip + comb * 128, &act, half * 64,
-                                        (x0 >> 7) * comb, 0, y0 + dy, b,
+                            tma_5d_pair(abase + st * strip + sp.gap * 128, &act, half * 64,
+                                        sp.cols ? y0 + dy : (x0 >> 7) * sp.fold, 0,
+                                        sp.cols ? 0 : y0 + dy, b,
                                         leader_addr(&sh.afull[st]));
                         else
                             tma_4d_pair(abase + st * strip, &act, half * 64, x0 + dx,
@@ -495,8 +503,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
             const uint32_t strip16 = strip >> 4;
             // rows of a strip: a tap's shift (a multiple of 128 bytes; the
             // 128-byte swizzle goes by address, so any row may come first)
-            const int shift = kComb ? comb : d;
-            const uint32_t row0 = sign > 0 ? 0 : (kTaps - 1) * (uint32_t)shift * 8;
+            const int shift = kComb ? sp.step : d;
+            const uint32_t row0 = (kComb ? sp.gap - sp.step : 0) * 8 +
+                                  (sign > 0 ? 0 : (kTaps - 1) * (uint32_t)shift * 8);
             const int rowstep = sign * shift * 8;
             const bool leader = elect_one();
             int it = 0, ast = 0, ag = 0;
@@ -566,10 +575,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
             const int tile = 2 * pr + rank, m = warp * 32 + lane;
             size_t p = (size_t)tile * 128 + m;
             if (kComb) {
-                // tile of the row: its tooth; pixel m: tooth m / comb, then m mod comb
-                const int r = tile >> (lgS - 7), c = tile & ((S >> 7) - 1);
-                const int tooth = m / comb;
-                p = ((size_t)r << lgS) + tooth * d + c * comb + (m - tooth * comb);
+                // a comb's first pixel: its row's, then its tooth's
+                const size_t first = sp.cols ? (size_t)tile * 128
+                                             : ((size_t)(tile >> (lgS - 7)) << lgS) +
+                                                   (tile & ((S >> 7) - 1)) * sp.fold;
+                const int q = m / sp.fold;
+                p = first + q * sp.outer + (m - q * sp.fold) * sp.inner;
             }
             uint32_t mask[64];
             if (kMode == kDgrad) {
@@ -1073,33 +1084,65 @@ bool map_act(CUtensorMap *m, const uint16_t *ptr, int n, int S, int pix = 128)
 // 84.5 us a layer at 8 x 256 x 256; three strips of 192 pixels, d = 32, took 126
 // and a box per tap, d = 64, 135).  Combs stream 128 pixels per strip whatever d
 // and fit three or four from d = 32 on (85.8 and 110 us); their teeth are 128 d
-// / S pixels wide and whole 1 KB groups.
+// / S pixels wide and whole 1 KB groups.  Columns do the same for S < 128 while
+// d < S (SMALL).
 StripShape conv_shape(int S, int d)
 {
-    StripShape sp{3, 128 + (2 * d + 7) / 8 * 8, 0, 0};
-    if (S >= 128) {
-        sp.na = std::min(4, kStripRoom / (sp.px * 128));
-        const int tooth = 128 * d / S;
-        if (sp.na < 4 && d < S && tooth >= 8) {
-            const int na = std::min(4, (kStripRoom - tooth * 128) / ((128 + tooth) * 128));
-            if (na >= 3 && na >= sp.na) return StripShape{3, 128 + tooth, na, tooth};
+    StripShape sp{};
+    sp.taps = 3;
+    const auto gapped = [&](int step) {   // stages between gaps of >= step pixels
+        sp.step = step;
+        sp.gap = (step + 7) / 8 * 8;
+        sp.px = 128 + sp.gap;
+        sp.na = std::min(4, (kStripRoom - sp.gap * 128) / (sp.px * 128));
+    };
+    if (S < 128) {
+        const int rows = 128 / S;
+        gapped(d * rows);
+        sp.fold = rows;
+        sp.outer = 1;
+        sp.inner = S;
+        sp.cols = 1;
+        if (d < S && sp.na >= 3) return sp;
+    } else {
+        const int tooth = 128 * d / S, px = 128 + (2 * d + 7) / 8 * 8;
+        const int na = std::min(4, kStripRoom / (px * 128));
+        if (na < 4 && d < S && tooth >= 8) {
+            gapped(tooth);
+            sp.fold = tooth;
+            sp.outer = d;
+            sp.inner = 1;
+            if (sp.na >= 3 && sp.na >= na) return sp;
         }
-        if (sp.na >= 3) return sp;
+        sp = StripShape{};
+        sp.taps = 3;
+        sp.px = px;
+        sp.na = na;
+        if (na >= 3) return sp;
     }
-    return StripShape{1, 128, kMaxA, 0};
+    sp = StripShape{};
+    sp.taps = 1;
+    sp.px = 128;
+    sp.na = kMaxA;
+    return sp;
 }
 
-// NHWC activations of 128 channels with x split into (x mod d, x / d): box 64
-// channels x w pixels x all S / d multiples of one row.
-bool map_comb(CUtensorMap *m, const uint16_t *ptr, int n, int S, int d, int w)
+// NHWC activations of 128 channels for a gapped strip: combs split x into (x mod
+// d, x / d), box 64 channels x one tooth at all S / d multiples of one row;
+// columns take y before x, box 64 channels x 128 / S rows x S columns.
+bool map_gapped(CUtensorMap *m, const uint16_t *ptr, int n, int S, int d,
+                const StripShape &sp)
 {
     auto fn = encoder();
     if (!fn) return false;
-    const cuuint64_t dims[5] = {128, (cuuint64_t)d, (cuuint64_t)(S / d), (cuuint64_t)S,
-                                (cuuint64_t)n};
-    const cuuint64_t strides[4] = {256, (cuuint64_t)d * 256, (cuuint64_t)S * 256,
-                                   (cuuint64_t)S * S * 256};
-    const cuuint32_t box[5] = {64, (cuuint32_t)w, (cuuint32_t)(S / d), 1, 1};
+    const cuuint64_t row = (cuuint64_t)S * 256, img = (cuuint64_t)S * row;
+    const cuuint64_t N = (cuuint64_t)n, s = (cuuint64_t)S;
+    const cuuint64_t teeth = sp.cols ? s : (cuuint64_t)(S / d);
+    const cuuint64_t dims[5] = {128, sp.cols ? s : (cuuint64_t)d, teeth, sp.cols ? 1 : s, N};
+    const cuuint64_t strides[4] = {sp.cols ? row : 256,
+                                   sp.cols ? 256 : (cuuint64_t)d * 256,
+                                   sp.cols ? img : row, img};
+    const cuuint32_t box[5] = {64, (cuuint32_t)sp.fold, (cuuint32_t)teeth, 1, 1};
     const cuuint32_t es[5] = {1, 1, 1, 1, 1};
     return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<uint16_t *>(ptr), dims,
               strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
@@ -1193,7 +1236,7 @@ cudaError_t launch_conv_tma(int mode, const uint16_t *in, const uint16_t *w,
         return cudaErrorInvalidValue;
     const StripShape sp = conv_shape(S, d);
     CUtensorMap ma, mw;
-    if (!(sp.comb ? map_comb(&ma, in, n, S, d, sp.comb) : map_act(&ma, in, n, S, sp.px)) ||
+    if (!(sp.step ? map_gapped(&ma, in, n, S, d, sp) : map_act(&ma, in, n, S, sp.px)) ||
         !map_wts(&mw, w))
         return cudaErrorInvalidValue;
     Epi e{bias, hprev, out, head ? *head : HeadArgs{}};
@@ -1210,7 +1253,7 @@ cudaError_t launch_conv_tma(int mode, const uint16_t *in, const uint16_t *w,
         {k_conv_pair<1, kFwdHead, false>, k_conv_pair<3, kFwdHead, false>,
          k_conv_pair<3, kFwdHead, true>}};
     const Kernel kern = kerns[mode != 0 ? kDgrad : head ? kFwdHead : kFwd]
-                             [sp.comb ? 2 : sp.taps == 3 ? 1 : 0];
+                             [sp.step ? 2 : sp.taps == 3 ? 1 : 0];
     if (attr == cudaSuccess)
         attr = cudaFuncSetAttribute(
             kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kPairSmem);
@@ -1218,8 +1261,7 @@ cudaError_t launch_conv_tma(int mode, const uint16_t *in, const uint16_t *w,
     // S >= 16: whole pairs of 128-pixel tiles
     const int npairs = (int)((long long)n * S * S / 256);
     return launch_pdl(kern, dim3(2 * std::min(npairs, nsm / 2)), kPairThreads, kPairSmem, st,
-                      ma, mw, e, sp.px, sp.na, sp.comb, S, lgS, d, mode == 0 ? 1 : -1, npairs,
-                      err);
+                      ma, mw, e, sp, S, lgS, d, mode == 0 ? 1 : -1, npairs, err);
 }
 
 // Weight gradient, added into dw[128][9 cin] (FP32, cleared by the caller), and

@@ -242,12 +242,20 @@ __global__ void __launch_bounds__(256)
     pdl_wait();
     const int w = blockIdx.x * blockDim.x + threadIdx.x;
     float l0 = 0.0f, l1 = 0.0f;
-    if (w < nw)
-        for (int pp = w; 2 * pp < P; pp += nw) {
-            const float2 t = term[pp];
-            l0 += t.x * inv_count;
-            l1 += t.y * inv_count;
+    if (w < nw) {
+        // at most 16 pairs (nw = 8 ceil(P / 256)), all loaded before the sums
+        float2 t[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            const int pp = w + i * nw;
+            t[i] = 2 * pp < P ? term[pp] : make_float2(0.0f, 0.0f);
         }
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            l0 += t[i].x * inv_count;
+            l1 += t[i].y * inv_count;
+        }
+    }
     double l = (double)(l0 + l1);
     for (int o = 16; o; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
     __shared__ double red[8];
@@ -823,7 +831,8 @@ int fire_net_backward(fire_ctx *ctx, fire_net *net, int n, const uint16_t *x,
     CUDA_TRY(ctx, cudaMemsetAsync(net->loss, 0, 8, st), "loss clear");
     CUDA_TRY(ctx, cudaMemsetAsync(net->grad, 0, (size_t)kParams * 4, st), "grad clear");
     CUDA_TRY(ctx, net_forward(net, n, x, net->prob, target, err, st), "surrogate forward");
-    const int per = 256;
+    // pixels per block: fewer where 256 would leave SMs without a block or two
+    const int per = P >= (1 << 18) ? 256 : 64;
     const int nblk = (P + per - 1) / per;
     CUDA_TRY(ctx, launch_pdl(k_head_grad, dim3(nblk), 256, 0, st,
                              (const uint16_t *)net->h[kL - 1],
