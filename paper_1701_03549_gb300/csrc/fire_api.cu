@@ -188,6 +188,24 @@ int plan_launch(fire_ctx *ctx, int ntiles, long long n, LaunchPlan *p, bool burn
     return FIRE_OK;
 }
 
+// Launch shape and the state buffer of its blocks.  When the buffer cannot be
+// had, the shape that needs least of it: shared-memory state, or the fewest
+// blocks.  (A failure forced by fire_debug_fail_alloc is returned.)
+int plan_with_state(fire_ctx *ctx, int ntiles, long long n, LaunchPlan *p)
+{
+    const bool forced = ctx->fail_alloc_after >= 0;
+    int rc = FIRE_OK;
+    for (int lean = 0; lean < 2; ++lean) {
+        rc = plan_launch(ctx, ntiles, n, p, false, lean != 0);
+        if (rc || p->smem_state) return rc;
+        rc = grow_device(ctx, (void **)&ctx->gstate, &ctx->gstate_bytes,
+                         (size_t)p->grid * 2 * ntiles * 128, "simulation state");
+        if (rc != FIRE_ENOMEM || forced) return rc;
+        cudaGetLastError();   // the failed allocation's
+    }
+    return rc;
+}
+
 }  // namespace fire
 
 extern "C" {
@@ -511,16 +529,10 @@ int launch_batch(fire_ctx *ctx, const fire_map *m, int n,
 {
     const int ntiles = m->dev.ntiles;
     LaunchPlan plan;
-    int rc = plan_launch(ctx, ntiles, n, &plan);
+    int rc = plan_with_state(ctx, ntiles, n, &plan);
     if (rc) return rc;
     const bool smem_state = plan.smem_state;
     const long long grid = plan.grid;
-    if (!smem_state) {
-        const size_t need = (size_t)grid * 2 * ntiles * 128;
-        rc = grow_device(ctx, (void **)&ctx->gstate, &ctx->gstate_bytes, need,
-                         "simulation state");
-        if (rc) return rc;
-    }
     // longest-first processing order (scheduling only: every fire's result
     // depends on its own parameters, ignition and seed alone)
     const uint32_t *dorder = nullptr;

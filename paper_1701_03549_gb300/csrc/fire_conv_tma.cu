@@ -1085,7 +1085,7 @@ bool map_act(CUtensorMap *m, const uint16_t *ptr, int n, int S, int pix = 128)
 // and a box per tap, d = 64, 135).  Combs stream 128 pixels per strip whatever d
 // and fit three or four from d = 32 on (85.8 and 110 us); their teeth are 128 d
 // / S pixels wide and whole 1 KB groups.  Columns do the same for S < 128 while
-// d < S (SMALL).
+// d < S and three fit (32 x 32 x 32: 14.2 us a layer, 15.7 with a box per tap).
 StripShape conv_shape(int S, int d)
 {
     StripShape sp{};

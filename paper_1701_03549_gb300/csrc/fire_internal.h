@@ -280,6 +280,8 @@ int noalloc_take_error(int device, bool *set);
 // grown, so a state that fits in shared memory goes there).
 int plan_launch(fire_ctx *ctx, int ntiles, long long n, LaunchPlan *p,
                 bool burn = false, bool fixed_scratch = false);
+// plan_launch, with ctx->gstate grown for it (not for the burn-time variant).
+int plan_with_state(fire_ctx *ctx, int ntiles, long long n, LaunchPlan *p);
 // Launch that may begin while the kernel before it on the stream drains
 // (programmatic stream serialisation).  The kernel calls pdl_wait() before it
 // touches anything an earlier kernel wrote or reads; what comes before that

@@ -5,9 +5,9 @@
 // Simulation kernel design (one thread block per simulation at a time,
 // persistent blocks, the first simulation of each by its index and the next
 // ones from a global counter):
-//  * State: two bit planes X, Y (one bit per cell each) in 32 x 32-cell tiles,
-//    tile-major, in shared memory when they fit (else in a per-block global
-//    buffer).  A cell's 2-bit code is 00 burnable and unburnt, 11 burnt or
+//  * State: two bits X, Y per cell, one 8-byte pair of words per row of a
+//    32 x 32-cell tile, tile-major, in shared memory when they fit (else in a
+//    per-block global buffer).  A cell's 2-bit code is 00 burnable and unburnt, 11 burnt or
 //    non-burnable, and 10 / 01 burning, the code alternating with the parity
 //    of the step at which the cell ignited.  Within step t the sources are the
 //    cells coded "burning, parity t"; a tile's owner warp writes new cells
@@ -21,9 +21,11 @@
 //    tiles whose burning cells must be retired), deduplicated with per-tile
 //    mark bits; quiet tiles are never touched.  The fire is extinct when the
 //    list is empty.
-//  * Per tile (one warp, lane = tile row): eight bit masks of targets with a
-//    burning source in each direction, built with shifts across tile edges;
-//    the candidates are queued and spread evenly over the warp's lanes; each
+//  * Per tile (one warp, lane = tile row): the unburnt burnable cells with a
+//    source in the 3 x 3 window around them, across tile edges, are the
+//    candidates; each is queued with its direction mask, read from the three
+//    rows' three-cell windows through a byte table, by its row's lane or,
+//    in tiles with full rows, spread over the warp's lanes; each
 //    candidate draws one Philox block per half of its directions (counter =
 //    (cell, step, d/4, 0), key = seed) and decides the half's trials together
 //    through a fixed-point single-precision screen (float pairs where map or

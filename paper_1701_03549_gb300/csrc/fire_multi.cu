@@ -106,9 +106,6 @@ int fire_simulate_multi(fire_ctx *ctx, int nmaps, const fire_map *const *maps,
                                "non-burnable", i, g.row, g.col, mi);
         }
     }
-    LaunchPlan plan;
-    rc = plan_launch(ctx, ntiles_max, n, &plan);
-    if (rc) return rc;
 
     // map table and ranks (largest map first) on the device
     std::vector<MapDev> table(nmaps);
@@ -126,12 +123,9 @@ int fire_simulate_multi(fire_ctx *ctx, int nmaps, const fire_map *const *maps,
     rc = grow_device(ctx, &ctx->order, &ctx->order_bytes, ob + (size_t)n * 4,
                      "processing order");
     if (rc) return rc;
-    if (!plan.smem_state) {
-        rc = grow_device(ctx, (void **)&ctx->gstate, &ctx->gstate_bytes,
-                         (size_t)plan.grid * 2 * ntiles_max * 128,
-                         "simulation state");
-        if (rc) return rc;
-    }
+    LaunchPlan plan;
+    rc = plan_with_state(ctx, ntiles_max, n, &plan);
+    if (rc) return rc;
     // host-pointer arguments are staged (never under graph capture)
     const fire_params *dparams = params;
     const fire_cell *dign = ignitions;
