@@ -1157,7 +1157,7 @@ def run_surrogate(args):
         "roofline": {"bound": "tensor", "achieved": fwd_tflops, "peak": peak,
                      "unit": "TFLOP/s", "frac": fwd_tflops / peak,
                      "traffic": None, "kernel": "surrogate forward "
-                     "(k_conv_tma_p x7 + layer-1 k_conv1_tma + head), batch 8 x 256^2",
+                     "(k_conv_pair x7, head fused + layer-1 k_conv1), batch 8 x 256^2",
                      "peak_source": f"bf16_tflops ({kind})"},
         "cpu_baseline": None, "e2e": None, "gpu_launches": None,
         "clocks": ck,
@@ -1236,16 +1236,16 @@ def run_surrogate_step(args):
             "forward_ms": fwd_ms, "forward_tflops": fwd,
             "roofline": {"bound": "tensor", "achieved": trn, "peak": peak,
                          "unit": "TFLOP/s", "frac": trn / peak,
-                         "traffic": None, "kernel": "training step (k_conv_tma_p "
-                         "forward and input gradient, k_wgrad_tma, layer-1 "
-                         "tile, head, Adam)",
+                         "traffic": None, "kernel": "training step (k_conv_pair "
+                         "forward and input gradient, k_wgrad_strip, layer-1 "
+                         "k_conv1, head, Adam)",
                          "peak_source": f"bf16_tflops ({kind})"},
             "cpu_baseline": None, "e2e": None,
             # per training step: the forward pass (first layer + seven
-            # 128 -> 128 convolutions), head and head gradient, per layer a
-            # weight gradient and a bias gradient (8 each) and, above the
-            # first, an input gradient (7), and Adam
-            "gpu_launches": 34 * args.steps,
+            # 128 -> 128 convolutions, the head in the last one's epilogue),
+            # loss sum and head gradient, per layer a weight and bias gradient
+            # (8) and, above the first, an input gradient (7), and Adam
+            "gpu_launches": 26 * args.steps,
             "clocks": ck}))
     net.free()
     ctx.close()
