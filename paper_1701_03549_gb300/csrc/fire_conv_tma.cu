@@ -639,19 +639,23 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
 // with 16 all three rows (3 x N = 48); a column of ones beside them gives the
 // bias gradient in the same pass, shared out over the rows' CTAs.
 //
-// What bounds it (128 channels, 8 x 256 x 256, 154.6 GFLOP): the copies, 67 KB
-// per 128 pixels for 1536 clocks of MMAs (halving the MMAs saves a fifth), then
-// shared memory, which a 128 x 192 x 16 MMA reads at 107 bytes a clock.  90 us
-// with the bias (5 of them); one tap per CTA with a box per operand loaded 32 KB
-// per 64 pixels and tap: 119 us, and another 27 us for a bias pass over dz.  16
-// channels: 31 us (bound by reading dz, 134 MB) against 204 on register-staged
-// tiles.
+// What bounds it (128 channels, 8 x 256 x 256, 154.6 GFLOP): the copies into
+// shared memory, 64 to 72 KB per 128 pixels at 30 bytes a clock (1536 clocks of
+// MMAs; halving the MMAs saves a fifth, sharing dz by multicast within clusters of
+// three nothing), then shared memory, which a 128 x 192 x 16 MMA reads at 107 bytes
+// a clock.  Rows are taken in chains y, y + d, y + 2d, so that a row of `in` is read
+// by its three rows of taps one slab row apart and not d: 275 MB from DRAM instead
+// of 508 at d = 16, a training step 2075 us instead of 2095.  One tap per CTA with a box per
+// operand loaded 32 KB per 64 pixels and tap: 119 us, and another 27 us for a bias
+// pass over dz.  16 channels: 31 us (bound by reading dz, 134 MB) against 204 on
+// register-staged tiles.
 struct WgradShape {
     int L, lgw;        // pixels of a slab, log2 pixels of its rows
     int pitch;         // pixels from one row of a strip to the next
     int nbox, box;     // boxes of a strip and the bytes of one
     int tap;           // bytes from one tap to the next
     int strip, stages;
+    int lgm;           // log2 rows of a chain of rows d apart, 0: rows in order
 };
 
 constexpr int kMaxWgStages = 6;
@@ -740,7 +744,9 @@ __global__ void __launch_bounds__(kWgThreads, 1)
             if (leader) {
                 const int p0 = (s0 + s) * (kSteps * 16);
                 const int b = p0 >> (2 * lgS);
-                const int y = (p0 >> lgS) & (S - 1), x = p0 & (S - 1);
+                const int k = (p0 >> lgS) & (S - 1), x = p0 & (S - 1);
+                // 128 channels: row k of the order, y = k with lgm = 0
+                const int y = (k & ((1 << sp.lgm) - 1)) * d + (k >> sp.lgm);
                 const uint32_t sa = base + st * stage;
                 expect_tx(&sh.full[st], kDz + kB * sp.nbox * sp.box);
                 tma_4d(sa, &dzm, 0, x, y, b, &sh.full[st]);
@@ -1185,6 +1191,10 @@ WgradShape wgrad_shape(int S, int d, int cin)
         sp.tap = one ? d * row : sp.box;
         sp.strip = (sp.nbox * sp.box + 1023) / 1024 * 1024;
         sp.stages = std::min(kMaxWgStages, kWgRoom / (L * 256 + strips * sp.strip));
+        if (w == L && cin == 128) {   // chains of S / d rows
+            while ((d << (sp.lgm + 1)) <= S) ++sp.lgm;
+            if (d << sp.lgm != S) sp.lgm = 0;
+        }
         if (sp.stages >= 2 || L == 64) return sp;
     }
 }
