@@ -65,6 +65,17 @@ __device__ __forceinline__ void tma_4d(uint32_t dst, const CUtensorMap *map, int
         : "memory");
 }
 
+__device__ __forceinline__ void tma_5d(uint32_t dst, const CUtensorMap *map, int c0,
+                                       int c1, int c2, int c3, int c4, void *bar)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::"
+        "bytes [%0], [%1, {%2, %3, %4, %5, %6}], [%7];" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3),
+        "r"(c4), "r"(tc::smem_addr(bar))
+        : "memory");
+}
+
 __device__ __forceinline__ void tma_2d(uint32_t dst, const CUtensorMap *map, int c0,
                                        int c1, void *bar)
 {
@@ -640,15 +651,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
 // bias gradient in the same pass, shared out over the rows' CTAs.
 //
 // What bounds it (128 channels, 8 x 256 x 256, 154.6 GFLOP): the copies into
-// shared memory, 64 to 72 KB per 128 pixels at 30 bytes a clock (1536 clocks of
-// MMAs; halving the MMAs saves a fifth, sharing dz by multicast within clusters of
-// three nothing), then shared memory, which a 128 x 192 x 16 MMA reads at 107 bytes
-// a clock.  Rows are taken in chains y, y + d, y + 2d, so that a row of `in` is read
-// by its three rows of taps one slab row apart and not d: 275 MB from DRAM instead
-// of 508 at d = 16, a training step 2075 us instead of 2095.  One tap per CTA with a box per
-// operand loaded 32 KB per 64 pixels and tap: 119 us, and another 27 us for a bias
-// pass over dz.  16 channels: 31 us (bound by reading dz, 134 MB) against 204 on
-// register-staged tiles.
+// shared memory, 64 to 68 KB per 128 pixels at 30 bytes a clock for 1536 clocks
+// of MMAs (halving the MMAs saves a fifth; sharing dz by multicast in clusters of
+// three saves nothing and leaves 14 SMs idle), then shared memory, which a 128 x
+// 192 x 16 MMA reads at 107 bytes a clock.  Rows are taken in chains y, y + d, y +
+// 2d, so that the three rows of taps read a row of `in` one slab row apart and not
+// d: 275 MB from DRAM instead of 508 at d = 16, a training step 2075 us instead of
+// 2095; with combs 2060.  88 us a layer with the bias (d = 64, two stages: 96).
+// One tap per CTA with a box per operand loaded 32 KB per 64 pixels and tap: 119
+// us, and another 27 us for a bias pass over dz.  16 channels: 31 us (bound by
+// reading dz, 134 MB) against 204 on register-staged tiles.
 struct WgradShape {
     int L, lgw;        // pixels of a slab, log2 pixels of its rows
     int pitch;         // pixels from one row of a strip to the next
@@ -656,6 +668,7 @@ struct WgradShape {
     int tap;           // bytes from one tap to the next
     int strip, stages;
     int lgm;           // log2 rows of a chain of rows d apart, 0: rows in order
+    int fold;          // comb: pixels of a tooth, and of the gaps around the strip
 };
 
 constexpr int kMaxWgStages = 6;
@@ -716,6 +729,13 @@ __global__ void __launch_bounds__(kWgThreads, 1)
     }
     for (int i = tid; i < kOnesBytes / 4; i += kWgThreads)
         reinterpret_cast<uint32_t *>(sm + kWgRoom)[i] = 0x3f803f80u;
+    // zeros of the combs' gaps: no copy writes there
+    for (int i = tid; i < sp.stages * kB * 2 * sp.fold * 8; i += kWgThreads) {
+        const int gap = i / (sp.fold * 8), strip = gap >> 1;
+        unsigned char *const at = sm + (strip / kB) * stage + kDz + (strip % kB) * sp.strip +
+                                  (gap & 1) * (sp.strip - sp.fold * 128);
+        reinterpret_cast<uint4 *>(at)[i - gap * (sp.fold * 8)] = make_uint4(0, 0, 0, 0);
+    }
     tc::fence_proxy_async();
     if (tid == 0) {
         for (int i = 0; i < kMaxWgStages; ++i) {
@@ -749,9 +769,18 @@ __global__ void __launch_bounds__(kWgThreads, 1)
                 const int y = (k & ((1 << sp.lgm) - 1)) * d + (k >> sp.lgm);
                 const uint32_t sa = base + st * stage;
                 expect_tx(&sh.full[st], kDz + kB * sp.nbox * sp.box);
-                tma_4d(sa, &dzm, 0, x, y, b, &sh.full[st]);
-                tma_4d(sa + kDz / 2, &dzm, 64, x, y, b, &sh.full[st]);
-                for (int i = 0; i < kB; ++i) {
+                if (sp.fold) {
+                    const int xi = (x >> 7) * sp.fold, yi = y + (dyi - 1) * d;
+                    tma_5d(sa, &dzm, 0, xi, 0, y, b, &sh.full[st]);
+                    tma_5d(sa + kDz / 2, &dzm, 64, xi, 0, y, b, &sh.full[st]);
+                    const uint32_t in0 = sa + kDz + sp.fold * 128;
+                    tma_5d(in0, &inm, 0, xi, 0, yi, b, &sh.full[st]);
+                    tma_5d(in0 + sp.strip, &inm, 64, xi, 0, yi, b, &sh.full[st]);
+                } else {
+                    tma_4d(sa, &dzm, 0, x, y, b, &sh.full[st]);
+                    tma_4d(sa + kDz / 2, &dzm, 64, x, y, b, &sh.full[st]);
+                }
+                for (int i = 0; i < kB && !sp.fold; ++i) {
                     const int c = Cin == 128 ? 64 * i : 0;
                     const int yi = y + (Cin == 128 ? dyi - 1 : i - 1) * d;
                     for (int t = 0; t < sp.nbox; ++t)
@@ -1175,10 +1204,27 @@ bool map_nhwc(CUtensorMap *m, const uint16_t *ptr, int ch, int n, int S, int w, 
 }
 
 // Slabs and strips of the weight gradient: 128 pixels where two stages fit,
-// else 64.
+// else 64.  Rows of more than a slab are taken as combs (k_conv_pair) where the
+// teeth are whole 1 KB groups: 64 KB a slab whatever d, where strips of
+// neighbours take 32 KB + 256 (128 + 2 d) bytes (training step at S = 256: 2075 us
+// with strips, 2069 with combs of 16 pixels or more, 2060 with combs of 8).
 WgradShape wgrad_shape(int S, int d, int cin)
 {
     const int strips = cin == 128 ? 2 : 3, row = cin == 128 ? 128 : 32;
+    if (cin == 128 && S >= 256 && d < S && S % d == 0 && 128 * d / S >= 8) {
+        WgradShape sp{};
+        sp.L = 128;
+        sp.lgw = 7;
+        sp.fold = 128 * d / S;
+        sp.pitch = 128 + 2 * sp.fold;
+        sp.nbox = 1;
+        sp.box = 128 * 128;
+        sp.tap = sp.fold * 128;
+        sp.strip = sp.pitch * 128;
+        sp.stages = std::min(kMaxWgStages, kWgRoom / (128 * 256 + 2 * sp.strip));
+        while (d << sp.lgm < S) ++sp.lgm;
+        if (sp.stages >= 2) return sp;
+    }
     for (int L = 128;; L = 64) {
         WgradShape sp{};
         const int w = S < L ? S : L, R = L / w;
@@ -1289,8 +1335,11 @@ cudaError_t launch_wgrad_tma(const uint16_t *dz, const uint16_t *in, int cin, fl
     const WgradShape sp = wgrad_shape(S, d, cin);
     CUtensorMap mz, mi;
     const int w = 1 << sp.lgw;
-    if (!map_nhwc(&mz, dz, 128, n, S, w, sp.L / w) ||
-        !map_nhwc(&mi, in, cin, n, S, sp.pitch, sp.L / w))
+    StripShape comb{};
+    comb.fold = sp.fold;
+    if (sp.fold ? !map_gapped(&mz, dz, n, S, d, comb) || !map_gapped(&mi, in, n, S, d, comb)
+                : !map_nhwc(&mz, dz, 128, n, S, w, sp.L / w) ||
+                      !map_nhwc(&mi, in, cin, n, S, sp.pitch, sp.L / w))
         return cudaErrorInvalidValue;
     const bool eight = sp.L == 128;
     const auto kern = cin == 128 ? (eight ? k_wgrad_strip<128, 8> : k_wgrad_strip<128, 4>)
