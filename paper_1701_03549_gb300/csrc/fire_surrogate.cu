@@ -267,8 +267,6 @@ __global__ void __launch_bounds__(256)
     }
 }
 
-// dz of the top layer, head weight and bias gradients.  Block = 128 threads,
-// thread c = channel; each block walks `per` pixels.
 // Head gradient: dz[p, c] = g[p] wh[c] where h[p, c] > 0 (else 0), dwh[c] =
 // sum_p g[p] h[p, c], dwh[kC] = sum_p g[p]; threads as in k_bias_grad.
 __global__ void __launch_bounds__(256)
