@@ -31,7 +31,10 @@ constexpr int kFwd = 0, kDgrad = 1, kFwdHead = 2;
 
 struct Epi {
     const float *bias;        // forward
-    const uint16_t *hprev;    // input gradient: activations of the layer below
+    // [P][4] where activations are positive, channel c in bit (c % 32) / 2 + 16 (c
+    // % 2) of word c / 32: forward, of the output (nullable, written); input
+    // gradient, of the layer below
+    uint4 *bits;
     uint16_t *out;            // [P][128] BF16
     HeadArgs head;
 };
@@ -93,11 +96,6 @@ __device__ __forceinline__ uint32_t pack2(float a, float b)
     return *reinterpret_cast<const uint32_t *>(&h);
 }
 
-__device__ __forceinline__ bool pos16(uint32_t u)
-{
-    return !(u & 0x8000u) && (u & 0x7fffu);
-}
-
 // 32 bytes of one row per thread: whole sectors, where 16-byte accesses of
 // rows 256 bytes apart touch every sector twice.
 __device__ __forceinline__ void st_global32(void *p, const uint32_t v[8])
@@ -106,14 +104,6 @@ __device__ __forceinline__ void st_global32(void *p, const uint32_t v[8])
                  "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]),
                  "r"(v[6]), "r"(v[7])
                  : "memory");
-}
-
-__device__ __forceinline__ void ld_global32(const void *p, uint32_t v[8])
-{
-    asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]),
-                   "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
-                 : "l"(p));
 }
 
 // One lane of a converged warp.
@@ -320,15 +310,16 @@ __device__ __forceinline__ void head_pixel(const HeadArgs &hd, float bias,
 
 // Epilogue of one accumulator row (pixel p, 128 channels in tensor memory at
 // taddr): forward, bias and ReLU; input gradient, zero where the layer
-// below's activation (mask) is not positive; BF16 stores.  s_head: the head's
-// weights and bias.
+// below's activation is not positive (mask: its bits); BF16 stores.  s_head: the
+// head's weights and bias.
 template <int kMode>
 __device__ __forceinline__ void pair_epilogue(const Epi &epi, const float *s_bias,
                                               const float *s_head, uint32_t taddr,
-                                              size_t p, const uint32_t *mask)
+                                              size_t p, uint4 mask)
 {
     uint16_t *orow = epi.out + p * 128;
     float part[16];
+    uint32_t words[4] = {mask.x, mask.y, mask.z, mask.w};
 #pragma unroll
     for (int c0 = 0; c0 < 128; c0 += 32) {
         float v[32];
@@ -339,13 +330,18 @@ __device__ __forceinline__ void pair_epilogue(const Epi &epi, const float *s_bia
             for (int j = 0; j < 16; ++j)
                 pk[j] = pack2(fmaxf(v[2 * j] + s_bias[c0 + 2 * j], 0.0f),
                               fmaxf(v[2 * j + 1] + s_bias[c0 + 2 * j + 1], 0.0f));
-        } else {
+            if (epi.bits) {
+                uint32_t w = 0;   // a half that is not zero carries into its sign
 #pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                const uint32_t h = mask[c0 / 2 + j];
-                pk[j] = pack2(pos16(h & 0xffffu) ? v[2 * j] : 0.0f,
-                              pos16(h >> 16) ? v[2 * j + 1] : 0.0f);
+                for (int j = 0; j < 16; ++j)
+                    w |= (((pk[j] & 0x7fff7fffu) + 0x7fff7fffu) & 0x80008000u) >> (15 - j);
+                words[c0 / 32] = w;
             }
+        } else {
+            const uint32_t w = words[c0 / 32];
+#pragma unroll
+            for (int j = 0; j < 16; ++j)
+                pk[j] = pack2(v[2 * j], v[2 * j + 1]) & (((w >> j) & 0x10001u) * 0xffffu);
         }
         if (kMode == kFwdHead) {
 #pragma unroll
@@ -362,6 +358,8 @@ __device__ __forceinline__ void pair_epilogue(const Epi &epi, const float *s_bia
         st_global32(orow + c0, pk);
         st_global32(orow + c0 + 16, pk + 8);
     }
+    if (kMode != kDgrad && epi.bits)
+        epi.bits[p] = make_uint4(words[0], words[1], words[2], words[3]);
     if (kMode == kFwdHead) head_pixel(epi.head, s_head[128], part, p);
 }
 
@@ -593,12 +591,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
                 const int q = m / sp.fold;
                 p = first + q * sp.outer + (m - q * sp.fold) * sp.inner;
             }
-            uint32_t mask[64];
-            if (kMode == kDgrad) {
-#pragma unroll
-                for (int j = 0; j < 8; ++j)
-                    ld_global32(epi.hprev + p * 128 + 16 * j, mask + 8 * j);
-            }
+            const uint4 mask = kMode == kDgrad ? epi.bits[p] : make_uint4(0, 0, 0, 0);
             if (*(volatile int *)&sh.fail ||
                 !tc::mbar_wait_bounded(&sh.tfull[acc], (it >> 1) & 1)) {
                 atomicOr(&sh.fail, 1);
@@ -1056,7 +1049,8 @@ __global__ void __launch_bounds__(kC1Threads, 1)
             tc::fence_after_sync();
             pair_epilogue<kFwd>(epi, sh.bias, nullptr,
                                 tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * 128),
-                                (size_t)tile * 128 + q * 32 + lane, nullptr);
+                                (size_t)tile * 128 + q * 32 + lane,
+                                make_uint4(0, 0, 0, 0));
             tc::fence_before_sync();
             __syncwarp();
             if (lane == 0) mbar_arrive(&sh.tempty[acc]);
@@ -1278,12 +1272,13 @@ bool map_wts(CUtensorMap *m, const uint16_t *ptr)
 }  // namespace convtma
 
 // Forward (mode 0: out = ReLU(conv(in) + bias)) or input gradient (mode 1:
-// out = conv^T(in) masked by hprev > 0) of a 128 -> 128 layer over n samples
+// out = conv^T(in), zero where the layer below's bits are) of a 128 -> 128 layer
+// over n samples; forward with bits writes its own (Epi)
 // (head: forward only, the network's head on the result)
 // of S x S (S a power of two >= 16).  `w` is W[o][t][i] (forward) or
 // Wt[i][t][o] (input gradient), 16-byte aligned.
 cudaError_t launch_conv_tma(int mode, const uint16_t *in, const uint16_t *w,
-                            const float *bias, const uint16_t *hprev, uint16_t *out,
+                            const float *bias, uint4 *bits, uint16_t *out,
                             int n, int S, int lgS, int d, const HeadArgs *head,
                             uint32_t *err, cudaStream_t st)
 {
@@ -1295,7 +1290,7 @@ cudaError_t launch_conv_tma(int mode, const uint16_t *in, const uint16_t *w,
     if (!(sp.step ? map_gapped(&ma, in, n, S, d, sp) : map_act(&ma, in, n, S, sp.px)) ||
         !map_wts(&mw, w))
         return cudaErrorInvalidValue;
-    Epi e{bias, hprev, out, head ? *head : HeadArgs{}};
+    Epi e{bias, bits, out, head ? *head : HeadArgs{}};
     int dev = 0, nsm = 0;
     cudaError_t attr = cudaGetDevice(&dev);
     if (attr == cudaSuccess)
@@ -1362,8 +1357,8 @@ cudaError_t launch_wgrad_tma(const uint16_t *dz, const uint16_t *in, int cin, fl
 // First layer forward: out = ReLU(conv3x3(x, W1) + b1) for x [n][S][S][16]
 // and W1 [128][9][16] (BF16, 16-byte aligned), S a power of two >= 16.
 cudaError_t launch_conv1_tma(const uint16_t *x, const uint16_t *w, const float *bias,
-                             uint16_t *out, int n, int S, int lgS, uint32_t *err,
-                             cudaStream_t st)
+                             uint16_t *out, uint4 *bits, int n, int S, int lgS,
+                             uint32_t *err, cudaStream_t st)
 {
     using namespace convtma;
     if (S < 16 || (S & (S - 1)) || ((uintptr_t)x & 15) || ((uintptr_t)w & 15))
@@ -1373,7 +1368,7 @@ cudaError_t launch_conv1_tma(const uint16_t *x, const uint16_t *w, const float *
     const int bw = strips ? 130 : (S < 128 ? S : 128);
     if (!map_nhwc(&ma, x, 16, n, S, bw, strips ? 1 : 128 / bw) || !map_w144(&mw, w))
         return cudaErrorInvalidValue;
-    Epi e{bias, nullptr, out, HeadArgs{}};
+    Epi e{bias, bits, out, HeadArgs{}};
     const auto kern = strips ? k_conv1<3> : k_conv1<9>;
     const int smem = kC1Stages * (strips ? 3 * 5120 : 9 * kC1Tile) + 9 * kC1Tile + 2048;
     int dev = 0, nsm = 0;

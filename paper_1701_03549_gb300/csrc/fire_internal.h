@@ -314,11 +314,11 @@ struct HeadArgs {
     float *g, *term;
 };
 cudaError_t launch_conv_tma(int mode, const uint16_t *in, const uint16_t *w,
-                            const float *bias, const uint16_t *hprev, uint16_t *out,
+                            const float *bias, uint4 *bits, uint16_t *out,
                             int n, int S, int lgS, int d, const HeadArgs *head,
                             uint32_t *err, cudaStream_t st);
 cudaError_t launch_conv1_tma(const uint16_t *x, const uint16_t *w, const float *bias,
-                             uint16_t *out, int n, int S, int lgS, uint32_t *err,
+                             uint16_t *out, uint4 *bits, int n, int S, int lgS, uint32_t *err,
                              cudaStream_t st);
 cudaError_t launch_wgrad_tma(const uint16_t *dz, const uint16_t *in, int cin, float *dw,
                              float *db, int n, int S, int lgS, int d, uint32_t *err,

@@ -602,6 +602,7 @@ struct fire_net {
     uint16_t *wb = nullptr, *wt = nullptr;
     uint16_t *h[kL] = {};
     uint16_t *dz[kL] = {};
+    uint4 *bits[kL - 1] = {};   // where h is positive (training passes, S >= 16)
     float *prob = nullptr, *g = nullptr, *term = nullptr;
     double *loss = nullptr;
     int step = 0;
@@ -623,7 +624,7 @@ int ilog2(int v)
 
 // Forward over n <= max_batch samples of x: probabilities into prob, and with
 // target the loss (net->loss, cleared by the caller) and the per-pixel
-// gradient (net->g); activations stay in net->h.
+// gradient (net->g) and, for S >= 16, net->bits; activations stay in net->h.
 cudaError_t net_forward(fire_net *net, int n, const uint16_t *x, float *prob,
                         const float *target, uint32_t *err, cudaStream_t st)
 {
@@ -635,7 +636,7 @@ cudaError_t net_forward(fire_net *net, int n, const uint16_t *x, float *prob,
     cudaError_t e;
     if (S >= 16) {
         e = launch_conv1_tma(x, net->wb + w_off(0), net->theta + b_off(0), net->h[0],
-                             n, S, lgS, err, st);
+                             target ? net->bits[0] : nullptr, n, S, lgS, err, st);
         if (e != cudaSuccess) return e;
     } else {
         ConvFwd<kCin> p{x, net->wb + w_off(0), net->theta + b_off(0), net->h[0],
@@ -646,8 +647,9 @@ cudaError_t net_forward(fire_net *net, int n, const uint16_t *x, float *prob,
     for (int l = 1; l < kL; ++l) {
         if (S >= 16) {
             e = launch_conv_tma(0, net->h[l - 1], net->wb + w_off(l),
-                                net->theta + b_off(l), nullptr, net->h[l], n, S, lgS,
-                                kDil[l], l == kL - 1 ? &head : nullptr, err, st);
+                                net->theta + b_off(l),
+                                target && l < kL - 1 ? net->bits[l] : nullptr, net->h[l], n,
+                                S, lgS, kDil[l], l == kL - 1 ? &head : nullptr, err, st);
         } else {
             ConvFwd<kC> p{net->h[l - 1], net->wb + w_off(l), net->theta + b_off(l),
                           net->h[l], M, kC, 9 * kC, S, lgS, kDil[l]};
@@ -709,6 +711,8 @@ int fire_net_create(fire_ctx *ctx, int S, int max_batch, fire_net **out)
     size_t o_h[kL], o_dz[kL];
     for (int l = 0; l < kL; ++l) o_h[l] = take(pix * kC * 2);
     for (int l = 0; l < kL; ++l) o_dz[l] = take(pix * kC * 2);
+    size_t o_bits[kL - 1];
+    for (int l = 0; l < kL - 1; ++l) o_bits[l] = take(S >= 16 ? pix * 16 : 0);
     const size_t o_prob = take(pix * 4), o_g = take(pix * 4), o_term = take(pix * 4),
                  o_loss = take(8);
     cudaError_t e = cudaMalloc(&net->mem, off);
@@ -727,6 +731,7 @@ int fire_net_create(fire_ctx *ctx, int S, int max_batch, fire_net **out)
         net->h[l] = (uint16_t *)(b + o_h[l]);
         net->dz[l] = (uint16_t *)(b + o_dz[l]);
     }
+    for (int l = 0; l < kL - 1; ++l) net->bits[l] = (uint4 *)(b + o_bits[l]);
     net->prob = (float *)(b + o_prob);
     net->g = (float *)(b + o_g);
     net->term = (float *)(b + o_term);
@@ -862,7 +867,7 @@ int fire_net_backward(fire_ctx *ctx, fire_net *net, int n, const uint16_t *x,
         if (l > 0) {
             const uint16_t *wt = net->wt + (size_t)(l - 1) * kWl;
             if (S >= 16) {
-                CUDA_TRY(ctx, launch_conv_tma(1, net->dz[l], wt, nullptr, net->h[l - 1],
+                CUDA_TRY(ctx, launch_conv_tma(1, net->dz[l], wt, nullptr, net->bits[l - 1],
                                               net->dz[l - 1], n, S, lgS, kDil[l], nullptr,
                                               err, st), "input gradient");
             } else {
