@@ -380,9 +380,10 @@ __device__ __forceinline__ void pair_epilogue(const Epi &epi, const float *s_bia
 //    descriptor arithmetic per 64-wide slab it took 500 clocks a slab
 //    whatever the MMA count, against 256 for the slab's MMAs.  Waits and
 //    commits per row of taps, unrolled, leave the tensor core the bound.
-// Measured (one layer): 84.5 us for d <= 16 (1830 TFLOP/s) and, with combs, for
-// d = 32; 110 us for d = 64 (combs, three stages); the input gradients, which
-// also read the layer below's activations, 95 and 114.  One 128-pixel tile per
+// Measured (one layer): 84 us for d <= 16 (1840 TFLOP/s) and, with combs, for
+// d = 32; 108 us for d = 64 (combs, three stages); the input gradients 83 and 105
+// with the layer below's ReLU mask as bits, 96 and 114 when they read its
+// activations for it (32 KB more into an SM per tile).  One 128-pixel tile per
 // CTA with boxes per tap and streamed weights took 136 us for every d, and 158
 // for the input gradients.
 //
