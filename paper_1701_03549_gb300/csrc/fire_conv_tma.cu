@@ -651,7 +651,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
 // 192 x 16 MMA reads at 107 bytes a clock.  Rows are taken in chains y, y + d, y +
 // 2d, so that the three rows of taps read a row of `in` one slab row apart and not
 // d: 275 MB from DRAM instead of 508 at d = 16, a training step 2075 us instead of
-// 2095; with combs 2060.  88 us a layer with the bias (d = 64, two stages: 96).
+// 2095; with combs 2060.  86 us a layer with the bias (d = 64, two stages: 92).
 // One tap per CTA with a box per operand loaded 32 KB per 64 pixels and tap: 119
 // us, and another 27 us for a bias pass over dz.  16 channels: 31 us (bound by
 // reading dz, 134 MB) against 204 on register-staged tiles.
