@@ -516,6 +516,9 @@ __global__ void k_expand(int n, int reps, const fire_params *__restrict__ gp,
 // --- screening --------------------------------------------------------------
 // Predicted Eq. 2 fitness with expected set sizes; a cluster of kSpread blocks
 // per candidate, whose partial sums meet in the first block's shared memory.
+// That memory may be stored to only once the first block runs: every block
+// arrives at the cluster's barrier as it begins and waits just before its
+// stores, which hides the arrival under the sums.
 // Bound by double-precision additions (five a cell at about two a clock and
 // SM): 35 us for 16 x 256 x 256, where one block per candidate, on 16 SMs, took
 // 149.
@@ -525,6 +528,7 @@ __global__ void __launch_bounds__(256)
                    const float *__restrict__ tfrac, double cells, int kind,
                    double *__restrict__ pred)
 {
+    if (kSpread > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
     const int s = blockIdx.x / kSpread, part = blockIdx.x % kSpread;
     const float *q = prob + (size_t)s * SS;
     double sq = 0.0, sqt = 0.0, st = 0.0;
@@ -540,6 +544,7 @@ __global__ void __launch_bounds__(256)
         st += __shfl_xor_sync(0xffffffffu, st, o);
     }
     __shared__ double red[3][8 * kSpread];
+    if (kSpread > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
     if ((threadIdx.x & 31) == 0) {
         const int w = part * 8 + (threadIdx.x >> 5);
         double *r = &red[0][w];
@@ -552,6 +557,7 @@ __global__ void __launch_bounds__(256)
         r[8 * kSpread] = sqt;
         r[16 * kSpread] = st;
     }
+    __syncwarp();   // the aligned barrier takes whole warps
     if (kSpread > 1)
         asm volatile("barrier.cluster.arrive.release.aligned;\n\t"
                      "barrier.cluster.wait.acquire.aligned;" ::: "memory");
