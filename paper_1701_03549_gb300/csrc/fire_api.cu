@@ -367,7 +367,7 @@ int fire_maps_upload(fire_ctx *ctx, int H, int W, float cell_m,
         (e = cudaMalloc(&m->blk, words * 4)) != cudaSuccess ||
         (e = cudaMalloc(&m->init, words * 8)) != cudaSuccess ||
         (e = cudaMalloc(&m->tgt, words * 4)) != cudaSuccess ||
-        (e = cudaMalloc(&m->tgt_count, 16)) != cudaSuccess) {
+        (e = cudaMalloc(&m->tgt_count, 32)) != cudaSuccess) {
         fire_map_free(m);
         return set_err(ctx, FIRE_ENOMEM, "map allocation: %s",
                        cudaGetErrorString(e));
@@ -411,24 +411,22 @@ int fire_maps_upload(fire_ctx *ctx, int H, int W, float cell_m,
         daspect = f[2];
         dwind = f[3];
     }
-    // the map's tgt_count words carry the covariates' flags (the wind varies, a
-    // cell is out of the fixed-point range) until the target is cleared below
+    // the map's tgt_count words carry the covariates' flags until the target is
+    // cleared below
     e = launch_features(H, W, dveg, delev, dslope, daspect, dwind, m->feat,
                         m->wdiag, m->cfl, m->tgt_count, ctx->stream);
-    uint32_t fl[2] = {1, 1};
-    float4 f0;
+    uint32_t fl[4] = {1, 1, 0, 0};
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(fl, m->tgt_count, sizeof fl, cudaMemcpyDeviceToHost,
                             ctx->stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(&f0, m->feat, sizeof f0, cudaMemcpyDeviceToHost,
-                            ctx->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
     if (e == cudaSuccess && !fl[1]) {
+        float wind[2];   // in range with every burnable cell, 0 without one
+        std::memcpy(wind, fl + 2, sizeof wind);
         m->dev.fx = 1;
         m->dev.uniform_wind = !fl[0];
-        m->dev.cw = (int)std::lrintf(f0.z * kFxOne);
-        m->dev.sw = (int)std::lrintf(f0.w * kFxOne);
+        m->dev.cw = (int)std::lrintf(wind[0] * kFxOne);
+        m->dev.sw = (int)std::lrintf(wind[1] * kFxOne);
         e = cudaMalloc(&m->fx, HW * (fl[0] ? sizeof(int4) : sizeof(int2)));
         if (e == cudaSuccess) {
             m->dev.fx2 = fl[0] ? nullptr : (const int2 *)m->fx;
@@ -444,7 +442,7 @@ int fire_maps_upload(fire_ctx *ctx, int H, int W, float cell_m,
     }
     if (e == cudaSuccess) e = launch_blocked(m->dev, dveg, m->blk, m->init, ctx->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(m->tgt, 0, words * 4, ctx->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(m->tgt_count, 0, 16, ctx->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(m->tgt_count, 0, 32, ctx->stream);
     // host copy of the burnable mask for validating host ignitions
     m->burnable_host.resize(HW);
     if (e == cudaSuccess) {

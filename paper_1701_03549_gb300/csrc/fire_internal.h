@@ -24,11 +24,12 @@ struct MapDev {
     int H, W, TH, TW, ntiles;
     const float4 *feat;         // (psi, sig, cos wind, sin wind) per cell
     const float2 *wdiag;        // cos(wind - 45 deg), cos(wind - 135 deg) per cell
-    // Fixed-point covariates of the simulation's screen (fx 0: some cell is out
-    // of their range and the float-pair screen runs).  A wind raster of one
-    // value everywhere (bit for bit) has the same cosine and sine in every
-    // cell: the simulation then reads them from here and only (psi, sig) per
-    // cell, 10 bytes with the flags; else (psi, sig, cos, sin), 18 bytes.
+    // Fixed-point covariates of the simulation's screen (fx 0: some burnable cell
+    // is out of their range and the float-pair screen runs).  A wind raster of
+    // one value in all burnable cells (bit for bit) has the same cosine and sine
+    // there: the simulation then reads them from here and only (psi, sig) per
+    // cell, 10 bytes with the flags; else (psi, sig, cos, sin), 18 bytes.  What
+    // cannot burn is never read, so it has no say in either.
     int fx, uniform_wind;
     int cw, sw;                 // scale 2^30, uniform wind
     const int2 *fx2;            // (psi, sig) per cell, uniform wind
@@ -135,6 +136,9 @@ __host__ __device__ inline SimLayout sim_layout(int ntiles, int qcap,
 }
 
 // Launchers (fire_kernels.cu).  All are asynchronous on `st`.
+// flags: [0] the wind varies among burnable cells; [1] a burnable cell is out of
+// the fixed-point range; [2], [3] cosine and sine (float bits) of the wind in the
+// first burnable cell; [4] that cell's index (~0: there is none).
 cudaError_t launch_features(int H, int W, const uint8_t *veg, const float *elev,
                             const float *slope, const float *aspect,
                             const float *wind, float4 *feat, float2 *wdiag,

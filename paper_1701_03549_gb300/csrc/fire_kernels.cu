@@ -67,7 +67,8 @@ __global__ void k_features(int H, int W, const uint8_t *__restrict__ veg,
                            uint32_t *__restrict__ flags)
 {
     const long long n = (long long)H * W;
-    const uint32_t wind0 = __float_as_uint(wind[0]);
+    const uint32_t first = flags[4];   // the first burnable cell
+    const uint32_t wind0 = first != 0xffffffffu ? __float_as_uint(wind[first]) : 0u;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x) {
         const int r = (int)(i / W), c = (int)(i - (long long)r * W);
@@ -92,11 +93,36 @@ __global__ void k_features(int H, int W, const uint8_t *__restrict__ veg,
         if (v == 1) f |= kFlagForest;
         if (v != 0) f |= kFlagBurnable;
         feat[i] = make_float4(psi, sig, cw, sw);
-        if (__float_as_uint(wind[i]) != wind0) flags[0] = 1u;
-        if (!fx_feature(psi, sig, cw, sw)) flags[1] = 1u;
+        if (v != 0) {
+            if (__float_as_uint(wind[i]) != wind0) flags[0] = 1u;
+            if (!fx_feature(psi, sig, cw, sw)) flags[1] = 1u;
+        }
+        if (i == (long long)first) {
+            flags[2] = __float_as_uint(cw);
+            flags[3] = __float_as_uint(sw);
+        }
         wdiag[i] = make_float2(__double2float_rn(spec::omega(cw, sw, 1)),
                                __double2float_rn(spec::omega(cw, sw, 3)));
         cfl[i] = f;
+    }
+}
+
+// Index of the first burnable cell into *first (~0 before): one block, which stops
+// at the first 16384 cells that hold one.
+__global__ void __launch_bounds__(1024)
+    k_first_burnable(long long n, const uint8_t *__restrict__ veg,
+                     uint32_t *__restrict__ first)
+{
+    for (long long c0 = 0; c0 < n; c0 += 16 * 1024) {
+        uint32_t best = 0xffffffffu;
+#pragma unroll
+        for (int k = 15; k >= 0; --k) {
+            const long long i = c0 + k * 1024 + threadIdx.x;
+            if (i < n && veg[i] != 0) best = (uint32_t)i;
+        }
+        best = __reduce_min_sync(kFull, best);
+        if ((threadIdx.x & 31) == 0 && best != 0xffffffffu) atomicMin(first, best);
+        if (__syncthreads_or(best != 0xffffffffu)) return;
     }
 }
 
@@ -1213,7 +1239,7 @@ __global__ void k_probabilities(MapDev m, const double *__restrict__ beta_dev,
     double b[5];
     for (int j = 0; j < 5; ++j) b[j] = beta_dev[j];
     const ScreenParams sp = screen_params(b);
-    const int k = m.fx ? fx_scale(b) : 0;
+    const int km = m.fx ? fx_scale(b) : 0;
     for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
          idx < 8 * HW; idx += (long long)gridDim.x * blockDim.x) {
         const int d = (int)(idx / HW);
@@ -1223,6 +1249,8 @@ __global__ void k_probabilities(MapDev m, const double *__restrict__ beta_dev,
         const bool forest = fl & kFlagForest, up = (fl >> d) & 1u;
         if (p32) {
             const float2 wd = m.wdiag[i];
+            // a cell that cannot burn may be out of range all the same
+            const int k = fx_feature(f.x, f.y, f.z, f.w) ? km : 0;
             p32[idx] = screen_any(b, sp, k, forest, f, wd.x, wd.y, up, d);
         }
         if (p64)
@@ -1401,8 +1429,10 @@ cudaError_t launch_features(int H, int W, const uint8_t *veg, const float *elev,
                             uint16_t *cfl, uint32_t *flags, cudaStream_t st)
 {
     const long long n = (long long)H * W;
-    cudaError_t e = cudaMemsetAsync(flags, 0, 2 * sizeof(uint32_t), st);
+    cudaError_t e = cudaMemsetAsync(flags, 0, 4 * sizeof(uint32_t), st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(flags + 4, 0xff, sizeof(uint32_t), st);
     if (e != cudaSuccess) return e;
+    k_first_burnable<<<1, 1024, 0, st>>>(n, veg, flags + 4);
     k_features<<<grid_for(n, 256), 256, 0, st>>>(H, W, veg, elev, slope, aspect,
                                                  wind, feat, wdiag, cfl, flags);
     return cudaGetLastError();
