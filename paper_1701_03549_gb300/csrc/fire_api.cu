@@ -188,9 +188,23 @@ int plan_launch(fire_ctx *ctx, int ntiles, long long n, LaunchPlan *p, bool burn
     return FIRE_OK;
 }
 
+// Whether the context's stream records a graph for its caller.
+bool capturing(fire_ctx *ctx)
+{
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(ctx->stream, &st) != cudaSuccess) {
+        cudaGetLastError();   // the legacy stream beside a capture elsewhere
+        return false;
+    }
+    return st != cudaStreamCaptureStatusNone;
+}
+
 // Launch shape and the state buffer of its blocks.  When the buffer cannot be
 // had, the shape that needs least of it: shared-memory state, or the fewest
-// blocks.  (A failure forced by fire_debug_fail_alloc is returned.)
+// blocks.  (A failure forced by fire_debug_fail_alloc is returned.)  Under a
+// capture a state that fits in shared memory goes there: nothing may be
+// allocated then, and a graph must not depend on a buffer that a later call
+// moves.
 int plan_with_state(fire_ctx *ctx, int ntiles, long long n, LaunchPlan *p)
 {
     const bool forced = ctx->fail_alloc_after >= 0;
@@ -198,6 +212,10 @@ int plan_with_state(fire_ctx *ctx, int ntiles, long long n, LaunchPlan *p)
     for (int lean = 0; lean < 2; ++lean) {
         rc = plan_launch(ctx, ntiles, n, p, false, lean != 0);
         if (rc || p->smem_state) return rc;
+        if (!lean && capturing(ctx)) {
+            rc = plan_launch(ctx, ntiles, n, p, false, true);
+            if (rc || p->smem_state) return rc;
+        }
         rc = grow_device(ctx, (void **)&ctx->gstate, &ctx->gstate_bytes,
                          (size_t)p->grid * 2 * ntiles * 128, "simulation state");
         if (rc != FIRE_ENOMEM || forced) return rc;
