@@ -43,23 +43,31 @@ int ensure_device(fire_ctx *ctx)
 }
 
 int grow_device(fire_ctx *ctx, void **buf, size_t *cap, size_t need,
-                const char *what)
+                const char *what, bool keep)
 {
     if (need <= *cap) return FIRE_OK;
-    ctx->epoch++;   // cached graphs may reference the old buffer
-    if (*buf) cudaFree(*buf);
-    *buf = nullptr;
-    *cap = 0;
-    size_t n = need + need / 4 + 256;
-    if (ctx->fail_alloc_after >= 0 && ctx->fail_alloc_after-- == 0)
+    const size_t n = need + need / 4 + 256;
+    const bool forced = ctx->fail_alloc_after >= 0 && ctx->fail_alloc_after-- == 0;
+    const auto release = [&] {
+        if (!*buf) return;
+        ctx->epoch++;   // cached graphs may reference the old buffer
+        cudaFree(*buf);
+        *buf = nullptr;
+        *cap = 0;
+    };
+    if (!keep || forced) release();
+    if (forced)
         return set_err(ctx, FIRE_ENOMEM, "cudaMalloc(%zu) for %s: failure "
                        "forced by fire_debug_fail_alloc", n, what);
-    cudaError_t e = cudaMalloc(buf, n);
+    void *fresh = nullptr;
+    cudaError_t e = cudaMalloc(&fresh, n);
     if (e != cudaSuccess) {
-        *buf = nullptr;
+        cudaGetLastError();   // not the next launch's
         return set_err(ctx, FIRE_ENOMEM, "cudaMalloc(%zu) for %s: %s", n, what,
                        cudaGetErrorString(e));
     }
+    release();
+    *buf = fresh;
     *cap = n;
     return FIRE_OK;
 }
@@ -199,29 +207,50 @@ bool capturing(fire_ctx *ctx)
     return st != cudaStreamCaptureStatusNone;
 }
 
-// Launch shape and the state buffer of its blocks.  When the buffer cannot be
-// had, the shape that needs least of it: shared-memory state, or the fewest
-// blocks.  (A failure forced by fire_debug_fail_alloc is returned.)  Under a
-// capture a state that fits in shared memory goes there: nothing may be
-// allocated then, and a graph must not depend on a buffer that a later call
-// moves.
+// Launch shape and the state buffer of its blocks.  Where the buffer cannot be
+// had, a shape that needs less of it: the state in shared memory, else as many
+// blocks as there is room for (they are persistent: any number runs the batch).
+// The buffer that the context holds is given up for a larger one only once per
+// size that fails, so that calls on a full device neither free and allocate it
+// again each time nor drop the captured graphs.  (A failure forced by
+// fire_debug_fail_alloc is returned.)  Under a capture a state that fits in
+// shared memory goes there: nothing may be allocated then, and a graph must not
+// depend on a buffer that a later call moves.
 int plan_with_state(fire_ctx *ctx, int ntiles, long long n, LaunchPlan *p)
 {
+    int rc = plan_launch(ctx, ntiles, n, p);
+    if (rc || p->smem_state) return rc;
+    LaunchPlan lean;
+    const auto shared_state = [&] {
+        rc = plan_launch(ctx, ntiles, n, &lean, false, true);
+        if (!rc && lean.smem_state) *p = lean;
+        return rc || p->smem_state;
+    };
+    if (capturing(ctx) && shared_state()) return rc;
+
     const bool forced = ctx->fail_alloc_after >= 0;
-    int rc = FIRE_OK;
-    for (int lean = 0; lean < 2; ++lean) {
-        rc = plan_launch(ctx, ntiles, n, p, false, lean != 0);
-        if (rc || p->smem_state) return rc;
-        if (!lean && capturing(ctx)) {
-            rc = plan_launch(ctx, ntiles, n, p, false, true);
-            if (rc || p->smem_state) return rc;
-        }
-        rc = grow_device(ctx, (void **)&ctx->gstate, &ctx->gstate_bytes,
-                         (size_t)p->grid * 2 * ntiles * 128, "simulation state");
-        if (rc != FIRE_ENOMEM || forced) return rc;
-        cudaGetLastError();   // the failed allocation's
+    const size_t per_block = (size_t)2 * ntiles * 128, need = p->grid * per_block;
+    const auto grow = [&](size_t bytes, bool keep) {
+        return grow_device(ctx, (void **)&ctx->gstate, &ctx->gstate_bytes, bytes,
+                           "simulation state", keep);
+    };
+    rc = grow(need, true);
+    if (rc != FIRE_ENOMEM || forced) return rc;
+    if (!ctx->gstate_refused || need < ctx->gstate_refused) {
+        rc = grow(need, false);
+        if (rc != FIRE_ENOMEM) return rc;
+        ctx->gstate_refused = need;
     }
-    return rc;
+    if (shared_state()) return rc;
+    size_t held = ctx->gstate_bytes / per_block;
+    for (size_t blocks = p->grid / 2; !held && blocks; blocks /= 2) {
+        rc = grow(blocks * per_block, false);
+        if (rc && rc != FIRE_ENOMEM) return rc;
+        held = ctx->gstate_bytes / per_block;
+    }
+    if (!held) return FIRE_ENOMEM;
+    p->grid = (int)std::min<size_t>(p->grid, held);
+    return FIRE_OK;
 }
 
 }  // namespace fire

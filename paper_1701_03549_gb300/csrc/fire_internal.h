@@ -237,6 +237,7 @@ struct fire_ctx {
     size_t staging_bytes = 0;
     uint32_t *gstate = nullptr;      // global-state simulation buffers
     size_t gstate_bytes = 0;
+    size_t gstate_refused = 0;       // smallest size that failed (0: none yet)
     void *host_pinned = nullptr;     // pinned bounce buffer
     size_t host_pinned_bytes = 0;
     void *table = nullptr;           // map table + map ranks (multi-map calls)
@@ -274,8 +275,9 @@ namespace fire {
 int set_err(fire_ctx *ctx, int code, const char *fmt, ...);
 int cuda_err(fire_ctx *ctx, cudaError_t e, const char *what);
 int ensure_device(fire_ctx *ctx);
+// keep: the old buffer stays until the new one is there, and if it cannot be had.
 int grow_device(fire_ctx *ctx, void **buf, size_t *cap, size_t need,
-                const char *what);
+                const char *what, bool keep = false);
 size_t round16(size_t x);
 bool valid_map(const fire_map *m);
 int noalloc_take_error(int device, bool *set);
