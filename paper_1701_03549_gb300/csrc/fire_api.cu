@@ -109,12 +109,21 @@ bool valid_map(const fire_map *m) { return m && m->ctx && m->feat; }
 // tiles) is worth it for at most one fire per SM (801 x 801, q = 7: 17.1 shared,
 // 13.4 in global memory with two blocks).  The burn-time variant has no shared
 // state (256 x 256, q = 4: 4.3 at 8 warps, 5.5 at 4; 512 x 512, q = 13: 29.0
-// and 28.3).
+// and 28.3).  From 5 to 12 fires per SM four blocks of 8 warps need a second round,
+// which pays where the launch is as long as fires that fill the map (512 x 512
+// generation, q = 6.7: 17.7, eight blocks of 4 warps 20.9; a few such fires, 1024 x
+// 1024, q = 4.6: 12.0 against 15.2); others are done sooner in one round of eight
+// (reference parameters: 256 x 256, q = 8: 1.32 against 1.84, 1024 x 1024, q = 5: 12.3
+// against 18.1; a few that fill the map, q = 8: 256 x 256 1.55 against 2.2, 640 x 640
+// 7.0 against 8.2).
+//
+// spreading (burn only): the fires of the batch that fill the map, by their
+// parameters (launch_long_burn).
 //
 // fixed_scratch: the caller cannot provide a state buffer per block, so a state
 // that fits in shared memory goes there.
 int plan_launch(fire_ctx *ctx, int ntiles, long long n, LaunchPlan *p, bool burn,
-                bool fixed_scratch)
+                bool fixed_scratch, long long spreading)
 {
     int warps = 0, bps = 0, queue = 0, state = FIRE_STATE_AUTO;
     const bool override = ctx->warps_per_block || ctx->blocks_per_sm ||
@@ -141,7 +150,11 @@ int plan_launch(fire_ctx *ctx, int ntiles, long long n, LaunchPlan *p, bool burn
     if (!override && !tuned && (burn || (ntiles > 64 && !fixed_scratch))) {
         const long long sms = ctx->num_sms;
         const size_t shared = sim_layout(ntiles, 4096, true).total;
-        if (n >= (burn ? 12 : 24) * sms && ntiles <= 1024) {
+        // fires that fill the map end the launch: many of them, or any beyond 64
+        // tiles and up to six fires per SM
+        const bool one_round = burn && 16 * spreading < n &&
+                               n > (spreading && ntiles > 64 ? 6 : 4) * sms;
+        if ((one_round || n >= (burn ? 12 : 24) * sms) && ntiles <= 1024) {
             warps = 4, bps = 8, queue = burn ? 3072 : 2048, state = FIRE_STATE_GLOBAL;
         } else if (n >= (burn ? 2 : 8) * sms) {
             warps = 8, bps = 4, queue = 3072, state = FIRE_STATE_GLOBAL;

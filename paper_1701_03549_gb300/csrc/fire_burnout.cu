@@ -105,17 +105,18 @@ extern "C" int fire_simulate_burnout(fire_ctx *ctx, const fire_map *m, int n,
         return rc;
     }
     uint32_t *dlong = (uint32_t *)ctx->burn_aux;
-    uint32_t *dany = dlong + nwords;
-    uint32_t hany = 0;
-    cudaError_t e0 = launch_long_burn(m->dev, db, dlong, dany, ctx->stream);
+    uint32_t *dstats = dlong + nwords;
+    uint32_t stats[2] = {0, 0};   // any such cell; fires that fill the map
+    cudaError_t e0 = launch_long_burn(m->dev, db, n, dp, dlong, dstats, ctx->stream);
     if (e0 == cudaSuccess)
-        e0 = cudaMemcpyAsync(&hany, dany, 4, cudaMemcpyDeviceToHost, ctx->stream);
+        e0 = cudaMemcpyAsync(stats, dstats, sizeof stats, cudaMemcpyDeviceToHost,
+                             ctx->stream);
     if (e0 == cudaSuccess) e0 = cudaStreamSynchronize(ctx->stream);
     if (e0 != cudaSuccess) {
         if (tmp) cudaFree(tmp);
         return cuda_err(ctx, e0, "long-burn plane");
     }
-    if (!hany) {
+    if (!stats[0]) {
         rc = launch_batch(ctx, m, n, dp, di, ds, max_steps, 0u, dout, dsteps,
                           nullptr);
         cudaError_t e = cudaSuccess;
@@ -136,7 +137,7 @@ extern "C" int fire_simulate_burnout(fire_ctx *ctx, const fire_map *m, int n,
     // the bit-plane simulation kernel with burn times: state, two "still
     // burning" planes and a fuel byte per cell in each block's global buffer
     LaunchPlan plan;
-    rc = plan_launch(ctx, m->dev.ntiles, n, &plan, true);
+    rc = plan_launch(ctx, m->dev.ntiles, n, &plan, true, false, stats[1]);
     if (rc) {
         if (tmp) cudaFree(tmp);
         return rc;

@@ -161,10 +161,12 @@ inline cudaError_t reset_counter(uint32_t *counter, long long grid, int n, cudaS
 {
     return grid < n ? cudaMemsetAsync(counter, 0, 4, st) : cudaSuccess;
 }
-// Tile-major bit plane of the cells whose burn time is 2 or more, and a flag
-// set when there is any (zeroed by the launcher).
-cudaError_t launch_long_burn(const MapDev &m, const uint8_t *burn_time,
-                             uint32_t *plane, uint32_t *any, cudaStream_t st);
+// Tile-major bit plane of the cells whose burn time is 2 or more; stats (zeroed by
+// the launcher): [0] there is such a cell, [1] the fires with b0 > 0, which spread
+// across the wind and against it likelier than not and so fill the map.
+cudaError_t launch_long_burn(const MapDev &m, const uint8_t *burn_time, int n,
+                             const fire_params *params, uint32_t *plane,
+                             uint32_t *stats, cudaStream_t st);
 // Words of one block's global state in the burn-time variant.
 inline size_t burn_block_words(int ntiles, long long HW)
 {
@@ -285,7 +287,8 @@ int noalloc_take_error(int device, bool *set);
 // state is always in global memory; fixed_scratch: no state buffer can be
 // grown, so a state that fits in shared memory goes there).
 int plan_launch(fire_ctx *ctx, int ntiles, long long n, LaunchPlan *p,
-                bool burn = false, bool fixed_scratch = false);
+                bool burn = false, bool fixed_scratch = false,
+                long long spreading = 0);
 // plan_launch, with ctx->gstate grown for it (not for the burn-time variant).
 int plan_with_state(fire_ctx *ctx, int ntiles, long long n, LaunchPlan *p);
 // Launch that may begin while the kernel before it on the stream drains

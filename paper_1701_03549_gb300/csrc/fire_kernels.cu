@@ -172,10 +172,16 @@ __global__ void k_pack_bits(int H, int W, int TW, int nwords,
 
 // Tile-major bit plane of the cells that burn two steps or more.
 __global__ void k_long_burn(int H, int W, int TW, int nwords,
-                            const uint8_t *__restrict__ bt,
-                            uint32_t *__restrict__ dst, uint32_t *__restrict__ any)
+                            const uint8_t *__restrict__ bt, int n,
+                            const fire_params *__restrict__ params,
+                            uint32_t *__restrict__ dst, uint32_t *__restrict__ stats)
 {
     const int w = blockIdx.x * blockDim.x + threadIdx.x;
+    uint32_t c = 0;
+    for (long long i = w; i < n; i += (long long)gridDim.x * blockDim.x)
+        c += params[i].b[0] > 0.0;
+    c = __reduce_add_sync(kFull, c);
+    if ((threadIdx.x & 31) == 0 && c) atomicAdd(&stats[1], c);
     if (w >= nwords) return;
     const int k = w >> 5, r = w & 31;
     const int ti = k / TW, tj = k - ti * TW;
@@ -186,7 +192,7 @@ __global__ void k_long_burn(int H, int W, int TW, int nwords,
         if (R < H && C < W && bt[(long long)R * W + C] >= 2) word |= 1u << i;
     }
     dst[w] = word;
-    if (word) *any = 1u;
+    if (word) stats[0] = 1u;
 }
 
 // ---------------------------------------------------------------------------
@@ -1492,14 +1498,15 @@ cudaError_t launch_simulate(const SimLaunch &a, bool smem_state, int nwarps,
     return cudaGetLastError();
 }
 
-cudaError_t launch_long_burn(const MapDev &m, const uint8_t *burn_time,
-                             uint32_t *plane, uint32_t *any, cudaStream_t st)
+cudaError_t launch_long_burn(const MapDev &m, const uint8_t *burn_time, int n,
+                             const fire_params *params, uint32_t *plane,
+                             uint32_t *stats, cudaStream_t st)
 {
     const int nw = m.ntiles * 32;
-    cudaError_t e = cudaMemsetAsync(any, 0, sizeof(uint32_t), st);
+    cudaError_t e = cudaMemsetAsync(stats, 0, 2 * sizeof(uint32_t), st);
     if (e != cudaSuccess) return e;
-    k_long_burn<<<(nw + 255) / 256, 256, 0, st>>>(m.H, m.W, m.TW, nw, burn_time,
-                                                 plane, any);
+    k_long_burn<<<(nw + 255) / 256, 256, 0, st>>>(m.H, m.W, m.TW, nw, burn_time, n,
+                                                 params, plane, stats);
     return cudaGetLastError();
 }
 
