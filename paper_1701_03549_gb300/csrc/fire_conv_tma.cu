@@ -881,7 +881,7 @@ __global__ void __launch_bounds__(kWgThreads, 1)
         if (warp < 4 && nbias > 0) {
             float v[16];
             tc::tmem_ld16(lanes + kBiasCol, v);
-            atomicAdd(db + warp * 32 + lane, v[0]);
+            atomicAdd(db + (blockIdx.y % kSumSlots) * kSums + warp * 32 + lane, v[0]);
         }
     } else if (sh.fail && tid == 0) {
         atomicOr(err, 1u);
@@ -1317,8 +1317,8 @@ cudaError_t launch_conv_tma(int mode, const uint16_t *in, const uint16_t *w,
 }
 
 // Weight gradient, added into dw[128][9 cin] (FP32, cleared by the caller), and
-// bias gradient, added into db[128], of a layer of cin = 16 or 128 input
-// channels: dz [n][S][S][128] and in [n][S][S][cin] BF16, S a power of two >=
+// bias gradient, added into db[128] of kSumSlots slots, of a layer of cin = 16 or
+// 128 input channels: dz [n][S][S][128] and in [n][S][S][cin] BF16, S a power of two >=
 // 16; the pixel range is split over the SMs.
 cudaError_t launch_wgrad_tma(const uint16_t *dz, const uint16_t *in, int cin, float *dw,
                              float *db, int n, int S, int lgS, int d, uint32_t *err,

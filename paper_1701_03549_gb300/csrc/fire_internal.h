@@ -326,6 +326,14 @@ cudaError_t launch_conv_tma(int mode, const uint16_t *in, const uint16_t *w,
                             const float *bias, uint4 *bits, uint16_t *out,
                             int n, int S, int lgS, int d, const HeadArgs *head,
                             uint32_t *err, cudaStream_t st);
+// Bias and head gradients are sums over all pixels.  An FP32 atomic addition rounds
+// the running total, so they are added in kSumSlots slots of kSums floats, a block's
+// partial sums into the slot of its number, and the slots together in double
+// precision at the end (k_round_sums).  Error against 64-bit sums of the same terms,
+// of the norm: 32 samples at S = 32, bias 2.9e-8 and head 3.5e-8 (one slot: 1.7e-7
+// and 3.4e-7); 8 at S = 256, 4.2e-7 (the tensor core's chains) and 5.0e-8 (4.6e-7 and
+// 6.5e-7).  The launch that adds them also hands out the loss, which was a copy.
+constexpr int kSums = FIRE_NET_LAYERS * 128 + 129, kSumSlots = 16;
 cudaError_t launch_conv1_tma(const uint16_t *x, const uint16_t *w, const float *bias,
                              uint16_t *out, uint4 *bits, int n, int S, int lgS, uint32_t *err,
                              cudaStream_t st);

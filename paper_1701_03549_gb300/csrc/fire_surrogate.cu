@@ -311,8 +311,25 @@ __global__ void __launch_bounds__(256)
         float sum = 0.0f;
 #pragma unroll
         for (int r = 0; r < 16; ++r) sum += red[r][threadIdx.x];
-        atomicAdd(dwh + threadIdx.x, sum);
+        atomicAdd(dwh + (blockIdx.x % kSumSlots) * kSums + threadIdx.x, sum);
     }
+}
+
+// Bias gradients of every layer and the head's gradient from their slots, and the
+// loss for the caller (nullable).
+__global__ void __launch_bounds__(256)
+    k_round_sums(const float *__restrict__ slots, float *__restrict__ grad,
+                 const double *__restrict__ loss, double *__restrict__ loss_out)
+{
+    pdl_wait();
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i == 0 && loss_out) *loss_out = *loss;
+    if (i >= kSums) return;
+    double s = 0.0;
+#pragma unroll
+    for (int k = 0; k < kSumSlots; ++k) s += slots[k * kSums + i];
+    const int l = i / kC, c = i - l * kC;
+    grad[i < kL * kC ? b_off(l) + c : kHead + (i - kL * kC)] = (float)s;
 }
 
 // Bias gradient: db[o] = sum_p dz[p, o].  A block of 256 threads takes
@@ -342,7 +359,7 @@ __global__ void __launch_bounds__(256)
         float sum = 0.0f;
 #pragma unroll
         for (int r = 0; r < 16; ++r) sum += red[r][threadIdx.x];
-        atomicAdd(db + threadIdx.x, sum);
+        atomicAdd(db + (blockIdx.x % kSumSlots) * kSums + threadIdx.x, sum);
     }
 }
 
@@ -610,7 +627,9 @@ struct fire_net {
     uint16_t *dz[kL] = {};
     uint4 *bits[kL - 1] = {};   // where h is positive (training passes, S >= 16)
     float *prob = nullptr, *g = nullptr, *term = nullptr;
+    // behind the gradient, cleared with it: the loss, then the slots
     double *loss = nullptr;
+    float *slots = nullptr;
     int step = 0;
 };
 
@@ -620,6 +639,10 @@ int net_err(fire_ctx *ctx, const char *what)
 {
     return set_err(ctx, FIRE_EINVAL, "%s", what);
 }
+
+// The gradient, and with the loss and the slots behind it.
+constexpr size_t kGradBytes = ((size_t)kParams * 4 + 15) / 16 * 16;
+constexpr size_t kGradClear = kGradBytes + 16 + 4 * (size_t)kSums * kSumSlots;
 
 int ilog2(int v)
 {
@@ -711,7 +734,7 @@ int fire_net_create(fire_ctx *ctx, int S, int max_batch, fire_net **out)
         off += (bytes + 255) & ~(size_t)255;
         return o;
     };
-    const size_t o_th = take(P * 4), o_gr = take(P * 4), o_m = take(P * 4),
+    const size_t o_th = take(P * 4), o_gr = take(kGradClear), o_m = take(P * 4),
                  o_v = take(P * 4), o_wb = take(P * 2),
                  o_wt = take((size_t)(kL - 1) * kWl * 2);
     size_t o_h[kL], o_dz[kL];
@@ -719,8 +742,7 @@ int fire_net_create(fire_ctx *ctx, int S, int max_batch, fire_net **out)
     for (int l = 0; l < kL; ++l) o_dz[l] = take(pix * kC * 2);
     size_t o_bits[kL - 1];
     for (int l = 0; l < kL - 1; ++l) o_bits[l] = take(S >= 16 ? pix * 16 : 0);
-    const size_t o_prob = take(pix * 4), o_g = take(pix * 4), o_term = take(pix * 4),
-                 o_loss = take(8);
+    const size_t o_prob = take(pix * 4), o_g = take(pix * 4), o_term = take(pix * 4);
     cudaError_t e = cudaMalloc(&net->mem, off);
     if (e != cudaSuccess) {
         delete net;
@@ -741,7 +763,8 @@ int fire_net_create(fire_ctx *ctx, int S, int max_batch, fire_net **out)
     net->prob = (float *)(b + o_prob);
     net->g = (float *)(b + o_g);
     net->term = (float *)(b + o_term);
-    net->loss = (double *)(b + o_loss);
+    net->loss = (double *)(b + o_gr + kGradBytes);
+    net->slots = (float *)(net->loss + 2);
     e = cudaMemsetAsync(net->mem, 0, o_h[0], ctx->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
     if (e != cudaSuccess) {
@@ -837,8 +860,7 @@ int fire_net_backward(fire_ctx *ctx, fire_net *net, int n, const uint16_t *x,
     cudaStream_t st = ctx->stream;
     uint32_t *err = ctx->counter + 1;
     const int S = net->S, lgS = net->lgS, P = n * S * S;
-    CUDA_TRY(ctx, cudaMemsetAsync(net->loss, 0, 8, st), "loss clear");
-    CUDA_TRY(ctx, cudaMemsetAsync(net->grad, 0, (size_t)kParams * 4, st), "grad clear");
+    CUDA_TRY(ctx, cudaMemsetAsync(net->grad, 0, kGradClear, st), "gradient clear");
     CUDA_TRY(ctx, net_forward(net, n, x, net->prob, target, err, st), "surrogate forward");
     // pixels per block: fewer where 256 would leave SMs without a block or two
     const int per = P >= (1 << 18) ? 256 : 64;
@@ -846,14 +868,14 @@ int fire_net_backward(fire_ctx *ctx, fire_net *net, int n, const uint16_t *x,
     CUDA_TRY(ctx, launch_pdl(k_head_grad, dim3(nblk), 256, 0, st,
                              (const uint16_t *)net->h[kL - 1],
                              (const float *)(net->theta + kHead), (const float *)net->g, P,
-                             per, net->dz[kL - 1], net->grad + kHead),
+                             per, net->dz[kL - 1], net->slots + kL * kC),
              "head gradient");
     const int kslabs = P / 64;
     for (int l = kL - 1; l >= 0; --l) {
         cudaError_t e;
         if (S >= 16) {
             e = launch_wgrad_tma(net->dz[l], l ? net->h[l - 1] : x, l ? kC : kCin,
-                                 net->grad + w_off(l), net->grad + b_off(l), n, S, lgS,
+                                 net->grad + w_off(l), net->slots + l * kC, n, S, lgS,
                                  kDil[l], err, st);
             CUDA_TRY(ctx, e, "weight gradient");
         } else {
@@ -867,7 +889,7 @@ int fire_net_backward(fire_ctx *ctx, fire_net *net, int n, const uint16_t *x,
                 e = tc::launch_tc_tile<128>(p, wgrad_split(9, kslabs), err, st);
             }
             CUDA_TRY(ctx, e, "weight gradient");
-            k_bias_grad<<<nblk, 256, 0, st>>>(net->dz[l], P, per, net->grad + b_off(l));
+            k_bias_grad<<<nblk, 256, 0, st>>>(net->dz[l], P, per, net->slots + l * kC);
             CUDA_TRY(ctx, cudaGetLastError(), "bias gradient");
         }
         if (l > 0) {
@@ -883,7 +905,12 @@ int fire_net_backward(fire_ctx *ctx, fire_net *net, int n, const uint16_t *x,
             }
         }
     }
-    if (loss)
+    const bool aligned = ((uintptr_t)loss & 7) == 0;
+    CUDA_TRY(ctx, launch_pdl(k_round_sums, dim3((kSums + 255) / 256), 256, 0, st,
+                             (const float *)net->slots, net->grad,
+                             (const double *)net->loss, aligned ? loss : nullptr),
+             "bias and head gradients");
+    if (!aligned)
         CUDA_TRY(ctx, cudaMemcpyAsync(loss, net->loss, 8, cudaMemcpyDeviceToDevice, st),
                  "loss out");
     if (flags & FIRE_SYNC) return fire_sync(ctx);
