@@ -374,8 +374,10 @@ __device__ __forceinline__ void pair_epilogue(const Epi &epi, const float *s_bia
 //    activations stream.  Distinct data reaches an SM from L2 at no more than
 //    about 30 bytes per clock when all SMs read (9 TB/s), and a 16 KB box per
 //    tap and half needs 64; a strip of 128 + 2 d pixels that serves the three
-//    taps of a row needs 6 to 8 KB per tap and half.  d = 64 has no room for
-//    three strips and streams a box per tap.
+//    taps of a row needs 6 to 8 KB per tap and half.  Wide dilations (32, 64) have
+//    no room for four such strips and take combs of 128 pixels (StripShape); where
+//    those can't be had (teeth below 8 pixels, or separate rows), three strips or a
+//    box per tap.
 //  * the issuing thread's own instructions: with waits, commits and
 //    descriptor arithmetic per 64-wide slab it took 500 clocks a slab
 //    whatever the MMA count, against 256 for the slab's MMAs.  Waits and
