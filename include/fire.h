@@ -155,9 +155,12 @@ FIRE_API int fire_sync(fire_ctx *ctx);
  * blocks per SM (0: as many as fit), candidate-queue entries per block
  * (0: default; at least 64) and state placement (FIRE_STATE_AUTO: shared
  * memory when the grid's state fits, else a per-block global buffer;
- * FIRE_STATE_SHARED; FIRE_STATE_GLOBAL).  Results do not depend on any of
- * them (see Trials above); a shape that does not fit the device makes the
- * next simulation call fail with FIRE_EINVAL. */
+ * FIRE_STATE_SHARED; FIRE_STATE_GLOBAL).  All four 0: the shape autotuned for
+ * the map's tile count, else one by the map and the batch.  Results do not
+ * depend on any of them (see Trials above); a shape that does not fit the
+ * device makes the next simulation call fail with FIRE_EINVAL.  Blocks whose
+ * state buffer cannot be allocated keep their state in shared memory where it
+ * fits, or run in smaller number; FIRE_ENOMEM when not even one can. */
 #define FIRE_STATE_AUTO 0
 #define FIRE_STATE_SHARED 1
 #define FIRE_STATE_GLOBAL 2
@@ -213,7 +216,11 @@ FIRE_API int fire_target_upload(fire_ctx *ctx, fire_map *map, const uint8_t *bur
  *                 set FIRE_STATUS_STEP_CAP.
  * Host ignitions that are outside the grid or non-burnable make the call
  * return FIRE_EIGNITION before any work is issued; a map uploaded through a
- * context on another device is refused with FIRE_EINVAL. */
+ * context on another device is refused with FIRE_EINVAL.
+ * With FIRE_DEVICE_PTRS and without FIRE_SYNC the call can be recorded by a
+ * stream capture of the caller's; a state that fits in shared memory (up to
+ * about 800 tiles) then goes there, and a larger one needs the buffer of an
+ * earlier call of that size, which must not move while the graph lives. */
 FIRE_API int fire_simulate_batch(fire_ctx *ctx, const fire_map *map, int n,
                         const fire_params *params, const fire_cell *ignitions,
                         const uint64_t *seeds, uint32_t max_steps,
@@ -231,7 +238,11 @@ FIRE_API int fire_simulate_batch(fire_ctx *ctx, const fire_map *map, int n,
  * array of 2 MiB that every GPU loading the library holds until the process
  * exits.  A map whose per-block state buffer does not fit in it (grids of
  * more than about 8191 tiles whose state also exceeds shared memory) is
- * rejected with FIRE_EINVAL before any work is issued.  The first call on a
+ * rejected with FIRE_EINVAL before any work is issued.  Blocks keep their
+ * state in shared memory where it fits, and beyond that as many run as the
+ * array holds buffers for: from 65 tiles on, with eight fires per SM or more,
+ * fire_simulate_batch's choice of more blocks with state in global memory is
+ * faster (801 x 801: one block per SM here).  The first call on a
  * device looks up the array's address once; make that first call before any
  * stream capture begins on the device.  All calls on a device share the
  * array and each clears its counter area before launching, so calls whose

@@ -105,7 +105,7 @@ bool valid_map(const fire_map *m) { return m && m->ctx && m->feat; }
 // eight blocks of 4 warps (512 x 512 generation, q = 27: 22.0 against 22.5 at 8
 // warps and 24.4 at 16; ignition search, q = 108: 46 against 54 and 75).  Up to
 // 64 tiles the shared-memory shapes stay within a few per cent of these.  A
-// shared-memory state of which only one block fits an SM (about 400 to 700
+// shared-memory state of which only one block fits an SM (about 380 to 820
 // tiles) is worth it for at most one fire per SM (801 x 801, q = 7: 17.1 shared,
 // 13.4 in global memory with two blocks).  The burn-time variant has no shared
 // state (256 x 256, q = 4: 4.3 at 8 warps, 5.5 at 4; 512 x 512, q = 13: 29.0
