@@ -408,6 +408,11 @@ __device__ __forceinline__ float screen_p(float z)
 // is exact up to 2^24 and 2^-24 relative above, as in the float-pair screen.
 // So p is within 1.2e-7 (6e-8) of z's share and 3.1e-7 + 0.23 2^-24 of the
 // exponential's and the reciprocal's: below kScreenErr0 whatever b3.
+// Measured against double precision, every cell and direction of a 333 x 517 map
+// with varying wind, 40 vectors each of Gauss(0, 5), Uniform[-30, 30] and around the
+// reference: largest 1.2e-7, 1.2e-7, 1.3e-7, root mean square 2.55e-8, 1.79e-8,
+// 2.17e-8; the float pairs 1.7e-7, 2.8e-7, 2.3e-7 and 2.57e-8, 1.95e-8, 2.34e-8 (they
+// hold z to 48 bits, but round it to one float and read rounded diagonal cosines).
 struct FxParams {
     long long K[2];   // b0 + b1 If, plus half a unit of the high word
     int b2, b4;
