@@ -532,13 +532,15 @@ __global__ void k_expand(int n, int reps, const fire_params *__restrict__ gp,
 
 // --- screening --------------------------------------------------------------
 // Predicted Eq. 2 fitness with expected set sizes; a cluster of kSpread blocks
-// per candidate, whose partial sums meet in the first block's shared memory.
-// That memory may be stored to only once the first block runs: every block
-// arrives at the cluster's barrier as it begins and waits just before its
-// stores, which hides the arrival under the sums.
-// Bound by double-precision additions (five a cell at about two a clock and
-// SM): 35 us for 16 x 256 x 256, where one block per candidate, on 16 SMs, took
-// 149.
+// per candidate, whose sums meet in the first block's shared memory.  That memory
+// may be stored to only once the first block runs: every block arrives at the
+// cluster's barrier as it begins and waits just before its stores, which hides the
+// arrival under the sums.
+// Bound by double-precision additions (five a cell at about two a clock and SM),
+// so a block's partial sums meet in a shared-memory tree, whose additions halve
+// with every step (a warp's shuffles add in all 32 lanes each time: 120 warp
+// additions a block against 36).  16 x 256 x 256: 30 us a call; one block per
+// candidate, on 16 SMs, takes 98.
 template <int kSpread>
 __global__ void __launch_bounds__(256)
     k_pred_fitness(int SS, const float *__restrict__ prob,
@@ -546,46 +548,45 @@ __global__ void __launch_bounds__(256)
                    double *__restrict__ pred)
 {
     if (kSpread > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
-    const int s = blockIdx.x / kSpread, part = blockIdx.x % kSpread;
+    const int s = blockIdx.x / kSpread, part = blockIdx.x % kSpread, tid = threadIdx.x;
     const float *q = prob + (size_t)s * SS;
     double sq = 0.0, sqt = 0.0, st = 0.0;
-    for (int c = part * blockDim.x + threadIdx.x; c < SS; c += kSpread * blockDim.x) {
+#pragma unroll 4
+    for (int c = part * 256 + tid; c < SS; c += kSpread * 256) {
         const double qc = q[c], tc_ = tfrac[c];
         sq += qc;
         sqt += qc * tc_;
         st += tc_;
     }
-    for (int o = 16; o; o >>= 1) {
-        sq += __shfl_xor_sync(0xffffffffu, sq, o);
-        sqt += __shfl_xor_sync(0xffffffffu, sqt, o);
-        st += __shfl_xor_sync(0xffffffffu, st, o);
+    __shared__ double red[3][256], parts[3][kSpread];
+    red[0][tid] = sq;
+    red[1][tid] = sqt;
+    red[2][tid] = st;
+    __syncthreads();
+    for (int n = 128; n > 0; n >>= 1) {
+        if (tid < n)
+            for (int k = 0; k < 3; ++k) red[k][tid] += red[k][tid + n];
+        __syncthreads();
     }
-    __shared__ double red[3][8 * kSpread];
-    if (kSpread > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-    if ((threadIdx.x & 31) == 0) {
-        const int w = part * 8 + (threadIdx.x >> 5);
-        double *r = &red[0][w];
-        if (kSpread > 1) {
-            uint64_t g;
-            asm volatile("mapa.u64 %0, %1, 0;" : "=l"(g) : "l"(r));
-            r = reinterpret_cast<double *>(g);
+    if (kSpread > 1) {
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        if (tid < 3) {
+            uint64_t to;
+            asm volatile("mapa.u64 %0, %1, 0;" : "=l"(to) : "l"(&parts[tid][part]));
+            *reinterpret_cast<double *>(to) = red[tid][0];
         }
-        r[0] = sq;
-        r[8 * kSpread] = sqt;
-        r[16 * kSpread] = st;
-    }
-    __syncwarp();   // the aligned barrier takes whole warps
-    if (kSpread > 1)
+        __syncwarp();   // the aligned barrier takes whole warps
         asm volatile("barrier.cluster.arrive.release.aligned;\n\t"
                      "barrier.cluster.wait.acquire.aligned;" ::: "memory");
-    else
-        __syncthreads();
-    if (part == 0 && threadIdx.x == 0) {
-        sq = sqt = st = 0.0;
-        for (int i = 0; i < 8 * kSpread; ++i) {
-            sq += red[0][i];
-            sqt += red[1][i];
-            st += red[2][i];
+    }
+    if (part == 0 && tid == 0) {
+        sq = red[0][0];
+        sqt = red[1][0];
+        st = red[2][0];
+        for (int i = 1; i < kSpread; ++i) {
+            sq += parts[0][i];
+            sqt += parts[1][i];
+            st += parts[2][i];
         }
         const double sim = cells * sq, inter = cells * sqt, tgt = cells * st;
         const double num = sim + tgt - 2.0 * inter;
