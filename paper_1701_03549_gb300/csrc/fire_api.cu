@@ -424,14 +424,14 @@ int fire_maps_upload(fire_ctx *ctx, int H, int W, float cell_m,
     if ((e = cudaMalloc(&m->feat, HW * sizeof(float4))) != cudaSuccess ||
         (e = cudaMalloc(&m->wdiag, HW * sizeof(float2))) != cudaSuccess ||
         (e = cudaMalloc(&m->cfl, HW * sizeof(uint16_t))) != cudaSuccess ||
-        (e = cudaMalloc(&m->blk, words * 4)) != cudaSuccess ||
-        (e = cudaMalloc(&m->init, words * 8)) != cudaSuccess ||
+        (e = cudaMalloc(&m->blk, words * 12)) != cudaSuccess ||   // and init
         (e = cudaMalloc(&m->tgt, words * 4)) != cudaSuccess ||
         (e = cudaMalloc(&m->tgt_count, 32)) != cudaSuccess) {
         fire_map_free(m);
         return set_err(ctx, FIRE_ENOMEM, "map allocation: %s",
                        cudaGetErrorString(e));
     }
+    m->init = (uint2 *)(m->blk + words);   // words: a multiple of 32
     m->dev.feat = m->feat;
     m->dev.wdiag = m->wdiag;
     m->dev.cfl = m->cfl;
@@ -532,7 +532,6 @@ void fire_map_free(fire_map *m)
     if (m->fx) cudaFree(m->fx);
     if (m->cfl) cudaFree(m->cfl);
     if (m->blk) cudaFree(m->blk);
-    if (m->init) cudaFree(m->init);
     if (m->tgt) cudaFree(m->tgt);
     if (m->tgt_count) cudaFree(m->tgt_count);
     delete m;
